@@ -3,25 +3,25 @@
 // One thread takes two pairs per 128-bit streaming load (evict-first, so the
 // pair stream does not push the pool out of L2), issued one round ahead.  It
 // first computes BH(bip) and looks the key (aip, BH(bip)) up in a
-// direct-mapped table of recently seen keys in shared memory: a pair whose
+// two-way table of recently seen keys in shared memory: a pair whose
 // key this block already handled in this launch sets exactly the same r
 // fields to the same values, so it is skipped (SetAT is idempotent within a
 // slice; a key pushed out of the table only means a repeat is processed
-// again).  Unseen keys go to a per-warp queue.  A pool larger than the L2
-// cache also has a key table in device memory shared by every block and
-// every ingest of the slice: every 32 queued keys, each lane claims one there
-// (one L2 access), and only keys new to the slice go on, through a second
-// per-warp queue, to Algorithm 3: each lane takes one, computes f(aip), the
-// frame, the r column indices and the ACT of the AT in registers, then sets the
-// r fields without reading them.  Without a key table the r words are read
-// together first, and a field that already holds the slice's value costs one
-// load and no atomic.  Across the 152 blocks a
-// hot key reaches the pool once instead of once per block, which spares r
-// DRAM sectors per repeat; with the pool in L2 a pool word costs what a claim
-// costs, so such pools have no key table.  The shared-memory table is 64 KB:
-// the rest of the SM's 256 KB of L1 / shared memory stays L1 cache, which
-// serves the pool words of keys the table missed (a 128 KB table ran 13 %
-// slower, a 192 KB one 2x slower).
+// again).  Unseen keys go to a per-warp queue.  Most pools also have a key
+// table in device memory shared by every block and every ingest of the slice:
+// every 32 queued keys, each lane claims one there (one L2 access), and only
+// keys new to the slice go on, through a second per-warp queue, to Algorithm 3:
+// each lane takes one, computes f(aip), the frame, the r column indices and the
+// ACT of the AT in registers, then sets the r fields without reading them.
+// Without a key table the r words are read together first, and a field that
+// already holds the slice's value costs one load and no atomic.  Across the
+// 152 blocks a hot key reaches the pool once instead of once per block.  What
+// bounds the launch is the number of requests the L2 serves (the link pool,
+// 92 MB: 12 M of them in 89 us, against 22 M in 103 us without a table; loads
+// mixed with atomics go at about 135 G a second there) and, for a pool in HBM,
+// DRAM's random accesses.  The seen table is 64 KB: with 128 KB the launch also
+// empties a larger table (6.2 -> 7.2 us for 65,536 pairs) and, where pool words
+// are read, leaves less L1 for them.
 #include <cooperative_groups.h>
 #include <cuda_runtime.h>
 
@@ -69,44 +69,45 @@ __device__ __forceinline__ uint32_t *field_word(const Params &P, uint32_t *pool,
 constexpr int INGEST_THREADS = 1024;
 constexpr int INGEST_WARPS = INGEST_THREADS / 32;
 constexpr int INGEST_BLOCKS_PER_SM = 1;
-constexpr uint32_t SEEN_LOG2 = 13;  // 8,192 keys = 64 KB of shared memory per block
+constexpr uint32_t SEEN_SETS_LOG2 = 13;  // 8,192 two-way sets of the seen table: 16,384 keys in 64 KB of shared memory per block
 constexpr uint32_t QCAP = 96;       // per-warp queue of keys new to the block (below 32 between rounds, + 64)
 constexpr uint32_t Q2CAP = 64;      // per-warp queue of keys new to the slice (below 32 between rounds, + 32)
-constexpr unsigned long long NO_KEY = ~0ull;  // BH values are < 2^16, so never a real key
+constexpr uint32_t NO_AIP = 0;      // marks an empty way; a pair of this address is never looked up
 
-__device__ __forceinline__ uint32_t seen_slot(uint32_t aip, uint32_t h)
-{
-    return (aip * 0x9E3779B1u ^ h * 0x85EBCA77u) >> (32 - SEEN_LOG2);
-}
-
-// True if (aip, h) was recorded in the table of seen keys; records it
-// otherwise.  Without CLUSTER: the block's own table.  With it: the 2^cl_log2
-// CTAs of a thread-block cluster share one table of 2^cl_log2 x 8,192 keys, each CTA holding
-// the keys whose hash picks it, reached by the others through distributed
-// shared memory; a key repeated across the cluster's SMs is then set once.
-// Plain loads and stores: two CTAs that both miss a key set it twice, which
-// only repeats an idempotent SetAT.
+// True if key (aip, h) was recorded in the table of seen keys; records it
+// otherwise.  The set is a hash of aip XOR an injective image of h (the table
+// has at least 2^12 sets and h < 4096), so the set and aip identify the key
+// exactly and a way holds the 32 bits of aip alone: twice the keys of 64-bit
+// entries.  Two ways, the newer first, the older pushed out.  By a model of the
+// tables, of the 33.5 M pairs of a slice of the long workload 10.1 M miss it
+// (11.5 M missed a direct-mapped table of 64-bit entries of the same 64 KB, and
+// 9.5 M would miss 128 KB); measured, the long ingest runs in 247 us (315 us
+// direct-mapped, 251 us with 128 KB), with slice counts in 374 us (382, 406).
+// Without CLUSTER: the block's own table.
+// With it: the 2^cl_log2 CTAs of a thread-block cluster share one table, each
+// CTA holding the sets whose top bits pick it, reached by the others through
+// distributed shared memory; a key repeated across the cluster's SMs is then
+// set once.  Plain loads and stores: two CTAs that both miss a key set it
+// twice, which only repeats an idempotent SetAT.
 template <bool CLUSTER>
-__device__ __forceinline__ bool seen_before(unsigned long long *seen, uint32_t aip, uint32_t h, uint32_t cl_log2)
+__device__ __forceinline__ bool seen_before(uint2 *seen, uint32_t aip, uint32_t h, uint32_t cl_log2)
 {
-    const unsigned long long key = ((unsigned long long)aip << 32) | h;
-    if constexpr (!CLUSTER) {
-        const uint32_t s = seen_slot(aip, h);
-        if (seen[s] == key)
-            return true;
-        seen[s] = key;
-        return false;
-    } else {
-        const uint32_t s_all = (aip * 0x9E3779B1u ^ h * 0x85EBCA77u) >> (32 - SEEN_LOG2 - cl_log2);
-        const uint32_t owner = s_all >> SEEN_LOG2, s = s_all & ((1u << SEEN_LOG2) - 1);
+    const uint32_t bits = SEEN_SETS_LOG2 + (CLUSTER ? cl_log2 : 0u);
+    uint32_t s = ((aip * 0x9E3779B1u) >> (32 - bits)) ^ ((h * 0x3C6EF373u) & ((1u << bits) - 1));
+    uint2 *t = seen;
+    if constexpr (CLUSTER) {
         namespace cg = cooperative_groups;
         cg::cluster_group cluster = cg::this_cluster();
-        unsigned long long *t = owner == cluster.block_rank() ? seen : cluster.map_shared_rank(seen, owner);
-        if (t[s] == key)
-            return true;
-        t[s] = key;
-        return false;
+        const uint32_t owner = s >> SEEN_SETS_LOG2;
+        s &= (1u << SEEN_SETS_LOG2) - 1;
+        if (owner != cluster.block_rank())
+            t = cluster.map_shared_rank(seen, owner);
     }
+    const uint2 e = t[s];
+    if (aip != NO_AIP && e.x == aip)
+        return true;
+    t[s] = make_uint2(aip, e.x);
+    return aip != NO_AIP && e.y == aip;
 }
 
 // L2 accesses to the key table carry the evict-last priority: the pool words
@@ -333,13 +334,13 @@ __global__ void __launch_bounds__(INGEST_THREADS, INGEST_BLOCKS_PER_SM)
     const uint64_t nvec = n / 2;
     const uint4 *__restrict__ pairs = reinterpret_cast<const uint4 *>(pairs_raw);
     const uint2 *__restrict__ tail = (n & 1) ? reinterpret_cast<const uint2 *>(pairs_raw + 2 * (n - 1)) : nullptr;
-    extern __shared__ unsigned long long seen[];
+    extern __shared__ uint2 seen[];
     const uint32_t lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     // the second queue only exists with a key table (its 16 KB otherwise stay L1 cache)
-    uint2 *queue = reinterpret_cast<uint2 *>(seen + (1u << SEEN_LOG2)) + warp * (QCAP + (P.keys ? Q2CAP : 0));
+    uint2 *queue = seen + (1u << SEEN_SETS_LOG2) + warp * (QCAP + (P.keys ? Q2CAP : 0));
     uint2 *q2 = queue + QCAP;
-    for (uint32_t i = threadIdx.x; i < (1u << SEEN_LOG2); i += blockDim.x)
-        seen[i] = NO_KEY;
+    for (uint32_t i = threadIdx.x; i < (1u << SEEN_SETS_LOG2); i += blockDim.x)
+        seen[i] = make_uint2(NO_AIP, NO_AIP);
     // every table of the cluster is empty before any CTA reaches into another's
     if constexpr (CLUSTER)
         cooperative_groups::this_cluster().sync();
@@ -415,7 +416,7 @@ cudaError_t launch_ingest(const Params &P, uint32_t w, uint32_t *pool, const uin
         return cudaSuccess;
     const uint64_t nvec = n / 2;
     *launches += 1;
-    const size_t smem = (sizeof(unsigned long long) << SEEN_LOG2) +
+    const size_t smem = (sizeof(uint2) << SEEN_SETS_LOG2) +
                         (size_t)INGEST_WARPS * (QCAP + (P.keys ? Q2CAP : 0)) * sizeof(uint2);
     return dispatch_w(w, [&](auto wb) {
         constexpr int WB = decltype(wb)::value;
