@@ -119,8 +119,9 @@ extern "C" {
  *          in the open slice (4 entries of 8 bytes per ATV, 1 to 32 MiB), so
  *          that a key repeated across the SMs reaches the pool once.  AUTO
  *          keeps one when the pool is larger than the device's L2 cache (the
- *          repeats then cost DRAM sectors); with the pool in L2 a pool word
- *          costs what a table entry costs.  Results are the same either way.
+ *          repeats then cost DRAM sectors), and, where the memory for it can
+ *          be had, for every other pool but those with slice counts and those
+ *          of a server.  Results are the same either way.
  *  cluster CTAs of a thread-block cluster that share one table of the keys
  *          their ingest has seen (each CTA's shared-memory table holds the
  *          keys that hash to it, reached by the others through distributed

@@ -32,8 +32,7 @@ struct Params {
     uint32_t xshift[8]; // 2W - c - s*i: shift of the doubled LBS giving x_i
     // Table of the (aip, BH(bip)) keys set in the open slice, shared by every
     // ingest block: 2^klg 64-bit entries, each a tag of the key and the low
-    // 32 bits of the slice (all ones = empty).  Null for a pool that fits in
-    // the L2 cache.
+    // 32 bits of the slice (all ones = empty).  Null for a pool without one.
     unsigned long long *keys;
     uint32_t klg;
     // ASSE_COUNTER_AT_HIST: per ATV, the ATs last set in each slice phase
@@ -101,8 +100,9 @@ inline bool byte_guard(uint32_t w, uint32_t counter, uint32_t k)
 }
 
 // Key table size for a pool of n_atv ATVs: 4 entries per ATV, 2^17 .. 2^22,
-// or none (0): with ASSE_KEYS_OFF, or with ASSE_KEYS_AUTO when the pool's
-// bytes fit in an L2 cache of l2_bytes.  (At least 2^17 entries keeps a tag
+// or none needed (0): with ASSE_KEYS_OFF, or with ASSE_KEYS_AUTO when the
+// pool's bytes fit in an L2 cache of l2_bytes (asse_create may keep one all
+// the same, of the size ASSE_KEYS_ON gives).  (At least 2^17 entries keeps a tag
 // below 2^31, so no entry is all ones.)
 inline uint32_t key_table_log2(unsigned long long n_atv, unsigned long long pool_bytes,
                                unsigned long long l2_bytes, uint32_t mode)
@@ -376,5 +376,8 @@ struct PoolBuffers {
 };
 PoolBuffers pool_buffers(asse_pool *p);
 uint64_t pool_device_bytes(const asse_config *cfg);
+// Whether key_table AUTO of cfg keeps a key table because the pool is larger
+// than the current device's L2 cache.
+bool pool_needs_keys(const asse_config *cfg);
 
 }  // namespace asse

@@ -63,6 +63,9 @@ asse_config pool_cfg(const asse_config *cfg)
 {
     asse_config c = *cfg;
     c.max_batch = 2;  // the server stages batches itself
+    // a key table that only makes the ingest faster is not charged to the budget, so none is kept
+    if (c.key_table == ASSE_KEYS_AUTO && !pool_needs_keys(&c))
+        c.key_table = ASSE_KEYS_OFF;
     return c;
 }
 
