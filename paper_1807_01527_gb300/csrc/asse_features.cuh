@@ -59,43 +59,11 @@ __device__ void feature_tables(const Params &P, uint32_t c0, uint32_t kp, RangeD
     }
 }
 
-template <int WB, int M = FEAT_MAXM>
-__device__ void atv_features(const Params &P, const uint32_t *wreg, const RangeDesc *desc, const uint32_t *actw,
-                             uint32_t kp, float lp, float lup, float lmean, uint16_t *hist, __nv_bfloat16 *row,
-                             uint32_t lane, uint32_t *cnt_out)
+// The feature row of one ATV of cnt active ATs whose ages are counted in hist
+// ([kp][32] 16-bit, a column per lane; left zero), by one warp.
+__device__ __forceinline__ void write_feature_row(const Params &P, uint32_t cnt, uint32_t kp, float lp, float lup,
+                                                  float lmean, uint16_t *hist, __nv_bfloat16 *row, uint32_t lane)
 {
-    constexpr uint32_t F = 32 / WB;
-    constexpr uint32_t FM = (1u << WB) - 1;
-    uint32_t cnt = 0;
-    const uint32_t nw = (P.g + F - 1) / F;
-#pragma unroll
-    for (int m = 0; m < M; m++) {
-        const uint32_t q = lane + 32u * m;
-        if (32u * m >= nw)
-            break;
-        if (q >= nw)
-            continue;
-        const uint32_t w = wreg[m];
-        uint32_t am = field_bits<WB>(w, desc[q]);
-        if (am == 0)
-            continue;
-        cnt += __popc(am);
-        const uint32_t acts = actw[q];
-        do {
-            const uint32_t j = __ffs(am) - 1;
-            am &= am - 1;
-            const uint32_t v = (w >> (j * WB)) & FM;
-            uint32_t age;
-            if (P.ace) {
-                age = P.k - v;  // a counter visited age slices ago holds k - age
-            } else {
-                age = ((acts >> (j * WB)) & FM) + P.k2 - v;  // (ACT of the AT's block - v) mod 2k
-                age = age >= P.k2 ? age - P.k2 : age;
-            }
-            hist[age * 32 + lane] += 1;
-        } while (am);
-    }
-    cnt = __reduce_add_sync(FULL_MASK, cnt);
     __syncwarp();
     uint32_t bins[2] = {0, 0};
 #pragma unroll
@@ -135,6 +103,46 @@ __device__ void atv_features(const Params &P, const uint32_t *wreg, const RangeD
             v = lmean;
         row[e] = __float2bfloat16_rn(v);
     }
+}
+
+template <int WB, int M = FEAT_MAXM>
+__device__ void atv_features(const Params &P, const uint32_t *wreg, const RangeDesc *desc, const uint32_t *actw,
+                             uint32_t kp, float lp, float lup, float lmean, uint16_t *hist, __nv_bfloat16 *row,
+                             uint32_t lane, uint32_t *cnt_out)
+{
+    constexpr uint32_t F = 32 / WB;
+    constexpr uint32_t FM = (1u << WB) - 1;
+    uint32_t cnt = 0;
+    const uint32_t nw = (P.g + F - 1) / F;
+#pragma unroll
+    for (int m = 0; m < M; m++) {
+        const uint32_t q = lane + 32u * m;
+        if (32u * m >= nw)
+            break;
+        if (q >= nw)
+            continue;
+        const uint32_t w = wreg[m];
+        uint32_t am = field_bits<WB>(w, desc[q]);
+        if (am == 0)
+            continue;
+        cnt += __popc(am);
+        const uint32_t acts = actw[q];
+        do {
+            const uint32_t j = __ffs(am) - 1;
+            am &= am - 1;
+            const uint32_t v = (w >> (j * WB)) & FM;
+            uint32_t age;
+            if (P.ace) {
+                age = P.k - v;  // a counter visited age slices ago holds k - age
+            } else {
+                age = ((acts >> (j * WB)) & FM) + P.k2 - v;  // (ACT of the AT's block - v) mod 2k
+                age = age >= P.k2 ? age - P.k2 : age;
+            }
+            hist[age * 32 + lane] += 1;
+        } while (am);
+    }
+    cnt = __reduce_add_sync(FULL_MASK, cnt);
+    write_feature_row(P, cnt, kp, lp, lup, lmean, hist, row, lane);
     if (cnt_out)
         *cnt_out = cnt;
     __syncwarp();

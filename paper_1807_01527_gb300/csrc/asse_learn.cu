@@ -121,89 +121,141 @@ struct SynthArgs {
     float bg_max;
 };
 
-// One block per state: the host's distinct bips and the background set the
-// ATs slice by slice (a later slice overwrites), the state is packed exactly
-// as ingest would have left it at the end of slice k-1, and its feature row
-// is computed from the packed words by atv_features.
-template <int WB>
-__global__ void __launch_bounds__(256) synth_kernel(Params P, SynthArgs S, uint64_t first, uint64_t n, bf16 *x,
-                                                    float *log_n, float *lc)
+constexpr int SYNTH_WARPS = 8;
+constexpr uint32_t SYNTH_MAX_BATCH = 32;      // states a block takes at a time
+constexpr uint32_t SYNTH_TABLE_BYTES = 49152; // largest table of mixed background draw indices
+
+// Shared memory of synth_kernel, in bytes.
+__host__ __device__ inline size_t synth_smem(uint32_t k, uint32_t g, uint32_t batch, bool table)
 {
-    constexpr uint32_t F = 32 / WB;
-    extern __shared__ uint32_t sm[];
-    int16_t *last = reinterpret_cast<int16_t *>(sm);                // [g]
-    uint32_t *words = sm + (P.g + 1) / 2;                           // [Wd]
-    uint32_t *hist_w = words + P.Wd;                                 // [64][32] 16-bit, kept zero between uses
-    uint16_t *hist = reinterpret_cast<uint16_t *>(hist_w);
-    RangeDesc *desc = reinterpret_cast<RangeDesc *>(hist_w + HIST_WORDS);  // [Wd]
-    uint32_t *actw = reinterpret_cast<uint32_t *>(desc + P.Wd);             // [Wd]
-    __shared__ uint32_t end[65];
-    __shared__ uint32_t card;
-    __shared__ float pbg;
-    const uint32_t tid = threadIdx.x;
-    for (uint32_t i = tid; i < HIST_WORDS; i += blockDim.x)
-        hist_w[i] = 0;
-    // the states are packed as of the end of slice k - 1 (block 0's ACT (k-1) mod 2k)
-    feature_tables<WB>(P, (P.k - 1) % P.k2, P.k, desc, actw);
-    __syncthreads();
-    for (uint64_t si = blockIdx.x; si < n; si += gridDim.x) {
-        const uint64_t key = splitmix(S.seed ^ splitmix(first + si + 0x51ED270B27ull));
-        if (tid == 0) {
+    return (size_t)batch * k * sizeof(double) + (table ? (size_t)k * g * sizeof(uint64_t) : 0) +
+           (size_t)SYNTH_WARPS * (g * sizeof(int) + k * 32 * sizeof(uint16_t)) +
+           (size_t)batch * (k + 1) * sizeof(uint32_t);
+}
+
+// The state at the end of slice k - 1 is, for every AT, the last slice that
+// set it, from two kinds of draws: the host's distinct bips, bip j in the
+// slice s with end[s] <= j < end[s + 1], and the background, which sets AT h
+// in slice s if its draw is below pbg.  All k slices are in the window, so
+// the age of an AT is k - 1 minus that slice and the packed words are not
+// needed.  What bounds it is integer issue, so the draws that cannot change
+// the state are not made:
+//  * the bips run from the last to the first, and once every AT is set the
+//    earlier ones (of the same or earlier slices) change nothing: about
+//    g ln g draws of up to 2^n_max_log2;
+//  * the background of an AT runs from the last slice back to its first hit,
+//    and only over slices after the bips'.  unit() < pbg is the same as the
+//    53-bit draw below ceil(pbg 2^53), an integer comparison, and the inner
+//    SplitMix64 of the draw index, the same for every state, comes from a
+//    table of the block where k g of them fit.
+// The FP64 terms (1/64 of the FP32 rate here) are computed with a lane per
+// state and slice, a batch of states at a time, then one warp draws one state.
+// 16,384 states of k = 10, g = 512, n up to 2^20: 2,290 us with a block a
+// state and every draw made, 200 us now.
+__global__ void __launch_bounds__(SYNTH_WARPS * 32) synth_kernel(Params P, SynthArgs S, uint64_t first, uint64_t n,
+                                                                 uint32_t batch, uint32_t visible, int table, bf16 *x,
+                                                                 float *log_n, float *lc)
+{
+    extern __shared__ double synth_sm[];
+    const uint32_t k = P.k, g = P.g;
+    double *w = synth_sm;                                              // [batch][k] shares, then their running sums
+    uint64_t *tab = reinterpret_cast<uint64_t *>(w + batch * k);       // [k][g] if table
+    int *last_all = reinterpret_cast<int *>(tab + (table ? k * g : 0));             // [warps][g]
+    uint16_t *hist_all = reinterpret_cast<uint16_t *>(last_all + SYNTH_WARPS * g);  // [warps][k][32], zero between uses
+    uint32_t *end_all = reinterpret_cast<uint32_t *>(hist_all + SYNTH_WARPS * k * 32);  // [batch][k + 1]
+    __shared__ uint32_t card[SYNTH_MAX_BATCH], cnts[SYNTH_MAX_BATCH];
+    __shared__ float pbg[SYNTH_MAX_BATCH];
+    __shared__ uint64_t below[SYNTH_MAX_BATCH];  // ceil(pbg 2^53)
+    const uint32_t tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    int *last = last_all + warp * g;
+    uint16_t *hist = hist_all + warp * k * 32;
+    for (uint32_t i = tid; i < SYNTH_WARPS * k * 32; i += blockDim.x)
+        hist_all[i] = 0;
+    if (table)
+        for (uint32_t i = tid; i < k * g; i += blockDim.x)
+            tab[i] = splitmix(((uint64_t)(i / g) << 32) | (i % g));
+    for (uint64_t b0 = (uint64_t)blockIdx.x * batch; b0 < n; b0 += (uint64_t)gridDim.x * batch) {
+        const uint32_t nb = (uint32_t)(n - b0 < batch ? n - b0 : batch);
+        auto state_key = [&](uint32_t q) { return splitmix(S.seed ^ splitmix(first + b0 + q + 0x51ED270B27ull)); };
+        for (uint32_t e = tid; e < nb * k; e += blockDim.x)
+            w[e] = -log(unit(state_key(e / k), 16 + e % k) + 1e-300);
+        for (uint32_t q = tid; q < nb; q += blockDim.x) {
+            const uint64_t key = state_key(q);
             const double lnmax = (double)S.n_max_log2 * 0.6931471805599453;
-            double c = floor(exp(unit(key, 1) * lnmax));
-            card = (uint32_t)(c < 1.0 ? 1.0 : c);
-            pbg = (float)(unit(key, 2) * (double)S.bg_max);
-            double tot = 0.0, w[64];
-            for (uint32_t s = 0; s < P.k; s++) {
-                w[s] = -log(unit(key, 16 + s) + 1e-300);
-                tot += w[s];
-            }
-            double cum = 0.0;
-            end[0] = 0;
-            for (uint32_t s = 0; s < P.k; s++) {
-                cum += w[s];
-                end[s + 1] = s + 1 == P.k ? card : (uint32_t)floor((double)card * cum / tot);
-            }
+            const double c = floor(exp(unit(key, 1) * lnmax));
+            card[q] = (uint32_t)(c < 1.0 ? 1.0 : c);
+            const float pb = (float)(unit(key, 2) * (double)S.bg_max);
+            pbg[q] = pb;
+            below[q] = (uint64_t)ceil((double)pb * 9007199254740992.0);
         }
-        for (uint32_t h = tid; h < P.g; h += blockDim.x)
-            last[h] = -1;
         __syncthreads();
-        const uint32_t base = (uint32_t)(key >> 32);
-        for (uint32_t s = 0; s < P.k; s++) {
-            for (uint32_t h = tid; h < P.g; h += blockDim.x)
-                if (unit(key ^ 0xB5ull, ((uint64_t)s << 32) | h) < (double)pbg)
-                    last[h] = (int16_t)s;
-            for (uint32_t j = end[s] + tid; j < end[s + 1]; j += blockDim.x)
-                last[bip_hash(P, mix32(base + j))] = (int16_t)s;
-            __syncthreads();
+        for (uint32_t q = tid; q < nb; q += blockDim.x) {
+            double cum = 0.0;
+            for (uint32_t s = 0; s < k; s++) {
+                cum += w[q * k + s];
+                w[q * k + s] = cum;
+            }
         }
-        // pack: an AT last set in slice s holds that slice's ACT (C0 = s)
-        for (uint32_t q = tid; q < P.Wd; q += blockDim.x) {
-            uint32_t wd = 0;
-            for (uint32_t j = 0; j < F; j++) {
-                const uint32_t pos = q * F + j;
-                if (pos < P.g) {
-                    const uint32_t h = pos_at(P, pos);  // the AT stored there
-                    const int s = last[h];
-                    const uint32_t v = s < 0 ? P.k2 : act_of(P, (uint32_t)s, act_block(P, h));
-                    wd |= v << (j * WB);
+        __syncthreads();
+        for (uint32_t e = tid; e < nb * k; e += blockDim.x) {
+            const uint32_t q = e / k, s = e - q * k;
+            uint32_t *end = end_all + q * (k + 1);
+            end[s + 1] = s + 1 == k ? card[q] : (uint32_t)floor((double)card[q] * w[e] / w[q * k + k - 1]);
+            if (s == 0)
+                end[0] = 0;
+        }
+        __syncthreads();
+        for (uint32_t q = warp; q < nb; q += SYNTH_WARPS) {
+            const uint64_t key = state_key(q);
+            const uint32_t base = (uint32_t)(key >> 32);
+            const uint32_t *end = end_all + q * (k + 1);
+            for (uint32_t h = lane; h < g; h += 32)
+                last[h] = -1;
+            __syncwarp();
+            // bips from the last to the first, 128 at a time, while an AT is unset
+            uint32_t unset = g, hi = card[q], s = k - 1;
+            while (hi > 0 && unset > 0) {
+                const uint32_t lo = hi > 128 ? hi - 128 : 0;
+                uint32_t fresh = 0;
+#pragma unroll
+                for (uint32_t u = 0; u < 4; u++) {
+                    if (lane + 32 * u < hi - lo) {
+                        const uint32_t j = hi - 1 - lane - 32 * u;
+                        while (end[s] > j)
+                            s--;
+                        fresh += atomicMax(&last[bip_hash(P, mix32(base + j))], (int)s) < 0 ? 1u : 0u;
+                    }
+                }
+                unset -= __reduce_add_sync(FULL_MASK, fresh);
+                hi = lo;
+            }
+            __syncwarp();
+            // background, and the ages counted in the lane's column
+            uint32_t cnt = 0;
+            const uint64_t bkey = key ^ 0xB5ull, lim = below[q];
+            for (uint32_t h = lane; h < g; h += 32) {
+                int l = last[h];
+                for (int t = (int)k - 1; t > l; t--) {
+                    const uint64_t ix = table ? tab[(uint32_t)t * g + h] : splitmix(((uint64_t)t << 32) | h);
+                    if ((splitmix(bkey ^ ix) >> 11) < lim)
+                        l = t;
+                }
+                if (l >= 0 && at_pos(P, h) < visible) {
+                    hist[(k - 1 - (uint32_t)l) * 32 + lane] += 1;
+                    cnt++;
                 }
             }
-            words[q] = wd;
+            cnt = __reduce_add_sync(FULL_MASK, cnt);
+            const float pw = 1.0f - powf(1.0f - pbg[q], (float)k);  // background activity over the window
+            write_feature_row(P, cnt, k, pw, powf(pw, (float)P.r), pw, hist, x + (b0 + q) * FEAT, lane);
+            if (lane == 0)
+                cnts[q] = cnt;
         }
         __syncthreads();
-        if (tid < 32) {
-            const float pw = 1.0f - powf(1.0f - pbg, (float)P.k);  // background activity over the window
-            uint32_t cnt = 0;
-            uint32_t wreg[FEAT_MAXM];
-            load_atv_words<WB>(P, words, tid, wreg);
-            atv_features<WB>(P, wreg, desc, actw, P.k, pw, powf(pw, (float)P.r), pw, hist, x + si * FEAT,
-                             tid, &cnt);
-            if (tid == 0) {
-                log_n[si] = (float)log((double)card);
-                const double c = cnt >= P.g ? (double)P.g - 0.5 : (double)cnt;
-                lc[si] = (float)(-(double)P.g * log(((double)P.g - c) / (double)P.g));
-            }
+        for (uint32_t q = tid; q < nb; q += blockDim.x) {
+            log_n[b0 + q] = (float)log((double)card[q]);
+            const double c = cnts[q] >= g ? (double)g - 0.5 : (double)cnts[q];
+            lc[b0 + q] = (float)(-(double)g * log(((double)g - c) / (double)g));
         }
         __syncthreads();
     }
@@ -604,18 +656,27 @@ int asse_synth_states(const asse_synth_cfg *cfg, uint64_t first, uint64_t n, uin
     const uint32_t Fw = 32 / w;
     P.Wd = ((cfg->g + Fw - 1) / Fw + 7) / 8 * 8;
     SynthArgs S{cfg->seed, cfg->n_max_log2, cfg->bg_max};
-    const size_t smem = ((cfg->g + 1) / 2 + P.Wd + HIST_WORDS) * sizeof(uint32_t) +
-                        (size_t)P.Wd * (sizeof(RangeDesc) + sizeof(uint32_t));
+    // ATVs of more than 933 words (g above 3,712 in byte-wide fields) are refused
+    if (P.Wd > 933)
+        return ASSE_ECUDA;
+    // a feature row counts the first 32 FEAT_MAXM words of an ATV, as the pool's kernels do
+    const uint32_t visible = 32 * FEAT_MAXM * Fw;
     int dev = 0, sms = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    const unsigned grid = (unsigned)(n < (uint64_t)sms * 8 ? n : (uint64_t)sms * 8);
-    cudaError_t e = dispatch_w(w, [&](auto wb) {
-        constexpr int WB = decltype(wb)::value;
-        synth_kernel<WB><<<grid, 256, smem, (cudaStream_t)stream>>>(P, S, first, n, reinterpret_cast<bf16 *>(x_dev),
-                                                                   log_n_dev, lc_dev);
-        return cudaGetLastError();
-    });
+    // as many states a block as leave four blocks an SM, 8 to 32 of them
+    const uint64_t share = n / ((uint64_t)sms * 4) / SYNTH_WARPS * SYNTH_WARPS;
+    const uint32_t batch = share < SYNTH_WARPS ? SYNTH_WARPS : share > SYNTH_MAX_BATCH ? SYNTH_MAX_BATCH : (uint32_t)share;
+    const bool table = (uint64_t)cfg->k * cfg->g * sizeof(uint64_t) <= SYNTH_TABLE_BYTES;
+    const size_t smem = synth_smem(cfg->k, cfg->g, batch, table);
+    const uint64_t blocks = (n + batch - 1) / batch;
+    cudaError_t e = cudaFuncSetAttribute(synth_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e == cudaSuccess) {
+        synth_kernel<<<(unsigned)(blocks < (1u << 30) ? blocks : (1u << 30)), SYNTH_WARPS * 32, smem,
+                       (cudaStream_t)stream>>>(P, S, first, n, batch, visible, table ? 1 : 0,
+                                               reinterpret_cast<bf16 *>(x_dev), log_n_dev, lc_dev);
+        e = cudaGetLastError();
+    }
     return e == cudaSuccess ? ASSE_OK : ASSE_ECUDA;
 }
 

@@ -255,3 +255,31 @@ def test_learned_estimate_with_fallback(mods):
         pool.restore()
         pool.advance()
         orc.advance()
+
+
+@pytest.mark.parametrize("k,g,n", [(1, 2, 1), (3, 31, 9), (10, 512, 33), (12, 512, 8), (13, 512, 7), (64, 1025, 25),
+                                   (31, 2560, 40)])
+def test_synth_states_from_their_draws(mods, k, g, n):
+    """Batches that end inside a block's, one and many slices, with and without
+    the table of draw indices (k g 8 up to 48 KB), hosts of one bip and of far
+    more than g: every AT's age is that of the last slice that drew it, so the
+    active counts are exact integers over g, rounded to BF16."""
+    asse, oracle, omlp, torch = mods
+    keys = synth.method_keys(2)
+    cfg = dict(k=k, g=g, r=4, n_max_log2=16, bg_max=0.05, seed=3, bh_a=keys["bh_a"], bh_b=keys["bh_b"])
+    x, ln, lc = (v.float().cpu().numpy() for v in asse.synth_states(cfg, 77, n))
+    inv = np.float32(1) / np.float32(g)
+    for si in range(n):
+        d = synth.training_state_draws(3, 77 + si, k, g, 16, 0.05)
+        last = np.full(g, -1)
+        for s in range(k):
+            with np.errstate(over="ignore"):
+                h = d["bips"][s].astype(np.uint64) * np.uint64(keys["bh_a"]) + np.uint64(keys["bh_b"])
+            last[((h >> np.uint64(32)) * np.uint64(g) >> np.uint64(32)).astype(np.int64)] = s
+            last[d["bg"][s]] = s
+        ages = np.bincount(k - 1 - last[last >= 0], minlength=64)[:64].astype(np.float32)
+        cnt = np.float32((last >= 0).sum())
+        np.testing.assert_array_equal(x[si, :65], _bf16(np.concatenate([[cnt], ages]) * inv), err_msg="state %d" % si)
+        assert ln[si] == np.float32(np.log(d["card"]))
+        want = -g * np.log((g - min(float(cnt), g - 0.5)) / g)
+        assert abs(lc[si] - want) <= 1e-6 * want + 1e-6
