@@ -127,18 +127,6 @@ __device__ __forceinline__ uint32_t act_of(const Params &P, uint32_t c0, uint32_
     return a >= P.k2 ? a - P.k2 : a;
 }
 
-// Algorithm 1 (AT) / aging-counter test (ACE) for one field value.
-__device__ __forceinline__ bool field_active(const Params &P, uint32_t v, uint32_t act, uint32_t kp)
-{
-    if (P.ace)
-        return v + kp >= P.k + 1;  // v >= k - k' + 1
-    if (v >= P.k2)
-        return false;
-    uint32_t dis = act + P.k2 - v;
-    dis = dis >= P.k2 ? dis - P.k2 : dis;
-    return dis + 1 <= kp;
-}
-
 // Algorithm 2 on one field whose new ACT is act (only 0 and k act).
 __device__ __forceinline__ uint32_t preserve(const Params &P, uint32_t v, uint32_t act)
 {
@@ -147,48 +135,6 @@ __device__ __forceinline__ uint32_t preserve(const Params &P, uint32_t v, uint32
     if (act == P.k)
         return (v == 0 || (v >= P.k && v < P.k2)) ? P.k2 : v;
     return v;
-}
-
-// Bit mask of the active fields of one packed word (bit j = field j),
-// fields at or past g excluded.
-template <int WB>
-__device__ __forceinline__ uint32_t active_fields(const Params &P, uint32_t word, uint32_t q, uint32_t c0,
-                                                  uint32_t kp)
-{
-    constexpr int F = 32 / WB;
-    constexpr uint32_t FM = (1u << WB) - 1;
-    const uint32_t h0 = q * F;
-    uint32_t am = 0;
-    if (P.ace) {
-#pragma unroll
-        for (int j = 0; j < F; j++) {
-            const uint32_t v = (word >> (j * WB)) & FM;
-            am |= (uint32_t)(v + kp >= P.k + 1) << j;
-        }
-    } else {
-        const uint32_t b0 = pos_block(P, h0), b1 = pos_block(P, h0 + F - 1);
-        if (b0 == b1) {
-            // one ACT for the whole word: active values are the cyclic window
-            // act, act-1, ..., act-k'+1 (mod 2k)
-            const uint32_t act = act_of(P, c0, b0);
-#pragma unroll
-            for (int j = 0; j < F; j++) {
-                const uint32_t v = (word >> (j * WB)) & FM;
-                uint32_t dis = act + P.k2 - v;
-                dis = dis >= P.k2 ? dis - P.k2 : dis;
-                am |= (uint32_t)((v < P.k2) & (dis < kp)) << j;
-            }
-        } else {
-#pragma unroll 1
-            for (int j = 0; j < F; j++) {
-                const uint32_t v = (word >> (j * WB)) & FM;
-                am |= (uint32_t)field_active(P, v, act_of(P, c0, pos_block(P, h0 + j)), kp) << j;
-            }
-        }
-    }
-    if (h0 + F > P.g)
-        am &= (P.g > h0) ? ((1u << (P.g - h0)) - 1) : 0u;
-    return am;
 }
 
 constexpr unsigned FULL_MASK = 0xffffffffu;

@@ -17,6 +17,7 @@
 #include <cstdint>
 
 #include "asse_device.cuh"
+#include "asse_swar.cuh"
 
 namespace asse {
 
@@ -259,38 +260,112 @@ __global__ void __launch_bounds__(RESTORE_THREADS) restore_kernel(Params P, Scan
     }
 }
 
-// Sec. 4.3 for given hosts: one warp per host; NAT as the AND over the r rows
-// of the active fields of each word, Eq. 4 with the frame's UP.
-template <int WB>
-__global__ void __launch_bounds__(256) estimate_kernel(Params P, const uint32_t *pool, uint32_t c0, uint32_t kp,
-                                                       const unsigned long long *aat, const uint32_t *aips,
-                                                       uint64_t n, asse_superpoint *out)
+constexpr int ESTIMATE_THREADS = 256;
+
+// Sec. 4.3 for given hosts: NAT as the AND over the r rows of the active
+// fields of each word, Eq. 4 with the frame's UP.
+//
+// A warp takes hpw hosts (4, 8, 16 or 32): lane l computes f of host l, then
+// eight lanes share a host, each reading 16-byte chunks of its r ATVs (r loads
+// in flight a lane) and testing them with the scan's range test, whose entry of
+// a word position, from a table of the block, serves all r rows.  NAT needs no
+// field order, so the guard bits of the rows are ANDed as they are.  Eq. 4
+// stays in FP64 (1/64 of the FP32 rate here: a lane per host keeps 32 of them
+// on one issue; with one lane of the warp at work it was most of the time) and
+// the UP of every frame is computed once per block.
+// A scan, a restore and the estimate of 100,003 hosts of a 92 MB pool (g = 512,
+// r = 4): 751 -> 215 us a pass, of which this kernel took 583.
+template <int WB, int R, bool BG>
+__global__ void __launch_bounds__(ESTIMATE_THREADS) estimate_kernel(Params P, const uint32_t *pool, uint32_t c0,
+                                                                    uint32_t kp, const unsigned long long *aat,
+                                                                    const uint32_t *aips, uint64_t n, uint32_t hpw,
+                                                                    asse_superpoint *out)
 {
-    constexpr uint32_t F = 32 / WB;
-    const int lane = threadIdx.x & 31;
-    const uint64_t warps = (uint64_t)gridDim.x * (blockDim.x / 32);
-    const uint32_t nwords = (P.g + F - 1) / F;
-    for (uint64_t t = (uint64_t)blockIdx.x * (blockDim.x / 32) + (threadIdx.x >> 5); t < n; t += warps) {
-        const uint32_t aip = aips[t];
-        const uint32_t f = mangle(P.A, aip);
-        const uint32_t z = f & (P.nf - 1);
-        const uint64_t LL = lbs_twice(P, f);
-        uint32_t nat = 0;
-        for (uint32_t q = lane; q < nwords; q += 32) {
-            uint32_t acc = FULL_MASK;
-            for (uint32_t i = 0; i < P.r; i++) {
-                const uint64_t atv = ((uint64_t)i << P.E_log2) + ((z << P.c) | column(P, LL, (int)i));
-                acc &= active_fields<WB>(P, pool[atv * P.Wd + q], q, c0, kp);
-            }
-            nat += __popc(acc);
+    extern __shared__ uint4 est_sm[];
+    uint4 *d_lo = est_sm;                                            // [Wd]
+    uint4 *d_hi = d_lo + P.Wd;                                       // [Wd], not for byte fields
+    double *up = reinterpret_cast<double *>(d_lo + (BG ? 1 : 2) * P.Wd);  // [nf]
+    for (uint32_t q = threadIdx.x; q < P.Wd; q += blockDim.x) {
+        if constexpr (BG) {
+            d_lo[q] = count_desc_bytes(P, q, c0, kp);
+        } else {
+            const RangeDesc d = count_desc<WB>(P, q, c0, kp);
+            d_lo[q] = make_uint4(d.lo1e, d.hih1e, d.lo1o, d.hih1o);
+            d_hi[q] = make_uint4(d.lo2e, d.hih2e, d.lo2o, d.hih2o);
         }
-        nat = __reduce_add_sync(FULL_MASK, nat);
-        if (lane == 0) {
+    }
+    for (uint32_t j = threadIdx.x; j < P.nf; j += blockDim.x)
+        up[j] = frame_up(P, aat, j);
+    __syncthreads();
+    const int r = R ? R : (int)P.r;
+    constexpr int RM = R ? R : 8;
+    const uint32_t lane = threadIdx.x & 31, sub = lane & 7, grp = lane >> 3;
+    const uint32_t chunks = P.Wd / 4;
+    const uint64_t stride = (uint64_t)gridDim.x * (ESTIMATE_THREADS / 32) * hpw;
+    for (uint64_t base = ((uint64_t)blockIdx.x * (ESTIMATE_THREADS / 32) + (threadIdx.x >> 5)) * hpw; base < n;
+         base += stride) {
+        const bool mine = lane < hpw && base + lane < n;
+        const uint32_t aip = mine ? aips[base + lane] : 0u;
+        const uint32_t f = mangle(P.A, aip);
+        uint32_t nat = 0;
+        for (uint32_t i0 = 0; i0 < hpw; i0 += 4) {
+            const uint32_t hf = __shfl_sync(FULL_MASK, f, i0 + grp);
+            uint32_t c = 0;
+            if (base + i0 + grp < n) {
+                const uint32_t z = hf & (P.nf - 1);
+                const uint64_t LL = lbs_twice(P, hf);
+                const uint4 *a[RM];
+#pragma unroll
+                for (int i = 0; i < RM; i++)
+                    if (i < r)
+                        a[i] = reinterpret_cast<const uint4 *>(
+                            pool + (((uint64_t)i << P.E_log2) + ((z << P.c) | column(P, LL, i))) * P.Wd);
+                for (uint32_t ch = sub; ch < chunks; ch += 8) {
+                    uint4 x[RM];
+#pragma unroll
+                    for (int i = 0; i < RM; i++)
+                        if (i < r)
+                            x[i] = a[i][ch];
+#pragma unroll
+                    for (int e = 0; e < 4; e++) {
+                        uint32_t m0 = FULL_MASK, m1 = FULL_MASK;
+                        if constexpr (BG) {
+                            const uint4 d = d_lo[4 * ch + e];
+#pragma unroll
+                            for (int i = 0; i < RM; i++)
+                                if (i < r)
+                                    m0 &= in_ranges_bytes(u4get(x[i], e), d);
+                            c += __popc(m0);
+                        } else {
+                            const RangeDesc d = load_desc(d_lo, d_hi, 4 * ch + e);
+#pragma unroll
+                            for (int i = 0; i < RM; i++) {
+                                if (i < r) {
+                                    uint32_t ev, od;
+                                    in_ranges<WB>(u4get(x[i], e), d, ev, od);
+                                    m0 &= ev;
+                                    m1 &= od;
+                                }
+                            }
+                            c += __popc(m0) + __popc(m1);
+                        }
+                    }
+                }
+            }
+            c += __shfl_xor_sync(FULL_MASK, c, 1);
+            c += __shfl_xor_sync(FULL_MASK, c, 2);
+            c += __shfl_xor_sync(FULL_MASK, c, 4);
+            // host i0 + g belongs to lane i0 + g
+            c = __shfl_sync(FULL_MASK, c, (lane & 3) * 8);
+            if ((lane & ~3u) == i0)
+                nat = c;
+        }
+        if (mine) {
             asse_superpoint sp;
             sp.aip = aip;
             sp.nat = nat;
-            eq4(P.g, P.theta, nat, frame_up(P, aat, z), sp.est, sp.flags);
-            out[t] = sp;
+            eq4(P.g, P.theta, nat, up[f & (P.nf - 1)], sp.est, sp.flags);
+            out[base + lane] = sp;
         }
     }
 }
@@ -312,12 +387,25 @@ cudaError_t launch_estimate(const Params &P, uint32_t w, const uint32_t *pool, u
 {
     if (n == 0)
         return cudaSuccess;
-    const uint64_t want = (n + 7) / 8;
-    const unsigned grid = (unsigned)(want > (uint64_t)sms * 8 ? (uint64_t)sms * 8 : want);
+    // as many hosts a warp as still leave eight warps an SM
+    uint32_t hpw = 32;
+    while (hpw > 4 && n < (uint64_t)hpw * sms * 8)
+        hpw /= 2;
+    const bool bg = byte_guard(w, P.ace ? ASSE_COUNTER_ACE : ASSE_COUNTER_AT, P.k);
+    const size_t smem = (size_t)(bg ? 1 : 2) * P.Wd * sizeof(uint4) + P.nf * sizeof(double);
     *launches += 1;
     return dispatch_w(w, [&](auto wb) {
         constexpr int WB = decltype(wb)::value;
-        estimate_kernel<WB><<<grid, 256, 0, s>>>(P, pool, c0, kp, aat, aips, n, out);
+        auto kern = P.r == 4 ? estimate_kernel<WB, 4, false> : estimate_kernel<WB, 0, false>;
+        if constexpr (WB == 8) {
+            if (bg)
+                kern = P.r == 4 ? estimate_kernel<8, 4, true> : estimate_kernel<8, 0, true>;
+        }
+        const uint64_t per = (uint64_t)hpw * (ESTIMATE_THREADS / 32);
+        const uint64_t want = (n + per - 1) / per;
+        const uint64_t full = (uint64_t)sms * resident_blocks(kern, ESTIMATE_THREADS, smem);
+        kern<<<(unsigned)(want < full ? want : full), ESTIMATE_THREADS, smem, s>>>(P, pool, c0, kp, aat, aips, n, hpw,
+                                                                                 out);
         return cudaGetLastError();
     });
 }
