@@ -48,7 +48,7 @@ TRAFFIC = {
 }
 KERNEL_SOURCES = {
     "ingest": ["asse_ingest.cu", "asse_device.cuh", "asse_internal.h"],
-    "scan": ["asse_scan.cu", "asse_swar.cuh", "asse_bytes.h", "asse_device.cuh", "asse_internal.h", "asse_ptx.cuh"],
+    "scan": ["asse_scan.cu", "asse_swar.cuh", "asse_cyclic.h", "asse_bytes.h", "asse_device.cuh", "asse_internal.h"],
     "hist_scan": ["asse_hist.cu", "asse_swar.cuh", "asse_bytes.h", "asse_device.cuh", "asse_internal.h"],
 }
 

@@ -51,8 +51,8 @@ extern "C" {
 #define ASSE_ECUDA 4     /* a CUDA runtime call or kernel launch failed */
 #define ASSE_ESTATE 5    /* call out of order (e.g. restore before scan) */
 /* 6 is ASSE_EAGAIN of asse_serve.h. */
-#define ASSE_ETIMEOUT 7  /* a bounded device-side wait gave up: a bulk copy or a
-                          * tensor-core pipeline stage did not complete within
+#define ASSE_ETIMEOUT 7  /* a bounded device-side wait gave up: a copy or a stage
+                          * of a tensor-core pipeline did not complete within
                           * about 2 s of SM clock.  The kernel returned instead
                           * of hanging and the CUDA context stays usable, but the
                           * outputs of that work are invalid (reload the pool
@@ -305,8 +305,7 @@ ASSE_API int asse_estimate(asse_pool *pool, const uint32_t *aips, uint64_t n, as
  * synchronises the stream.  Returns ECAPACITY if cap < count, or
  * if the restore overflowed restore_cap (then *n_out is the number of
  * column tuples the overflowing join level needed, a lower bound on the
- * capacity to configure, and out is not written).  Errors: ESTATE,
- * ETIMEOUT (a bounded wait of the scan gave up; the lists are invalid), ECUDA. */
+ * capacity to configure, and out is not written).  Errors: ESTATE, ECUDA. */
 ASSE_API int asse_report(asse_pool *pool, asse_superpoint *out, uint64_t cap, uint64_t *n_out, int where);
 
 /* As asse_report, but every restored candidate (CSIP, Algorithm 4), reported

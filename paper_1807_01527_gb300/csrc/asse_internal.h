@@ -136,8 +136,7 @@ struct Status {
     unsigned long long n_report;  // candidates with estimate >= theta
     unsigned long long needed;    // tuples the overflowing join level needed
     unsigned int overflow;        // a frame exceeded the restore capacity
-    unsigned int error;           // a device-side wait gave up (bounded mbarrier wait)
-    unsigned int pad[4];
+    unsigned int pad[5];
 };
 
 // A partial or complete column tuple of the restore join.
@@ -154,22 +153,6 @@ struct Refresh {
     uint32_t q_lo[2], q_hi[2];
     uint32_t n_ranges; // 0, 1 or 2 distinct word ranges
 };
-
-// Tile geometry of the scan kernel (asse_scan.cu).
-struct ScanGeom {
-    uint32_t lpa;         // lanes per ATV
-    uint32_t apt;         // ATVs per warp tile (32 / lpa)
-    uint32_t wseg;        // words per lane segment (Wd / lpa)
-    uint32_t seg_stride;  // shared-memory words per lane segment (odd number of 16-byte units)
-    uint32_t tile_words;  // 32 * seg_stride
-    uint32_t warps;       // warps per CTA that stream tiles
-    uint32_t tile_offset; // byte offset of the tile buffers in dynamic shared memory
-    uint32_t smem;        // dynamic shared memory bytes
-    uint32_t ilv;         // 1: interleaved chunks (lane p of an ATV owns its 16-byte chunks p, p + lpa, ...;
-                          //    the tile is apt whole ATVs back to back, one bulk copy); 0: lane segments
-};
-// nw windows: the count ranges of every window are kept in shared memory
-ScanGeom scan_geometry(uint32_t Wd, uint32_t mw, uint32_t nw, size_t smem_limit);
 
 // Slice-dependent launch arguments, kept in device memory so that a captured
 // CUDA graph replays unchanged from slice to slice: the open slice, the ACT

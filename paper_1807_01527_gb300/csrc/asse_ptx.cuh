@@ -1,5 +1,5 @@
-// Inline-PTX helpers shared by the kernels that stage data with bulk async
-// copies and mbarriers (scan) and by the tensor-core MLP (tcgen05, TMEM).
+// Inline-PTX helpers of the tensor-core MLP (tcgen05, TMEM), whose operands are
+// staged with bulk async copies and mbarriers, and of the wait probe.
 // Every wait is bounded: a wait that does not complete within WAIT_CYCLES
 // returns false and the caller records an error instead of hanging.
 #pragma once
@@ -60,21 +60,6 @@ __device__ __forceinline__ void bulk_load(void *dst, const void *src, uint32_t b
                      smem_addr(dst)),
                  "l"(src), "r"(bytes), "r"(smem_addr(bar))
                  : "memory");
-}
-
-// Shared -> global bulk copy in this thread's bulk group.
-__device__ __forceinline__ void bulk_store(void *dst, const void *src, uint32_t bytes)
-{
-    asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;" ::"l"(dst), "r"(smem_addr(src)),
-                 "r"(bytes)
-                 : "memory");
-    asm volatile("cp.async.bulk.commit_group;" ::: "memory");
-}
-
-// Until this thread's bulk stores have read their shared-memory source.
-__device__ __forceinline__ void bulk_store_drain()
-{
-    asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
 }
 
 // Order this thread's generic-proxy shared-memory accesses before later

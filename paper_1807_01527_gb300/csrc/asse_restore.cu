@@ -267,9 +267,9 @@ constexpr int ESTIMATE_THREADS = 256;
 //
 // A warp takes hpw hosts (4, 8, 16 or 32): lane l computes f of host l, then
 // eight lanes share a host, each reading 16-byte chunks of its r ATVs (r loads
-// in flight a lane) and testing them with the scan's range test, whose entry of
-// a word position, from a table of the block, serves all r rows.  NAT needs no
-// field order, so the guard bits of the rows are ANDed as they are.  Eq. 4
+// in flight a lane) and testing them with the scan's one-range test, whose entry
+// of a word position, from a table of the block, serves all r rows.  NAT needs
+// no field order, so the test's bits of the rows are ANDed as they are.  Eq. 4
 // stays in FP64 (1/64 of the FP32 rate here: a lane per host keeps 32 of them
 // on one issue; with one lane of the warp at work it was most of the time) and
 // the UP of every frame is computed once per block.
@@ -282,18 +282,13 @@ __global__ void __launch_bounds__(ESTIMATE_THREADS) estimate_kernel(Params P, co
                                                                     asse_superpoint *out)
 {
     extern __shared__ uint4 est_sm[];
-    uint4 *d_lo = est_sm;                                            // [Wd]
-    uint4 *d_hi = d_lo + P.Wd;                                       // [Wd], not for byte fields
-    double *up = reinterpret_cast<double *>(d_lo + (BG ? 1 : 2) * P.Wd);  // [nf]
-    for (uint32_t q = threadIdx.x; q < P.Wd; q += blockDim.x) {
-        if constexpr (BG) {
-            d_lo[q] = count_desc_bytes(P, q, c0, kp);
-        } else {
-            const RangeDesc d = count_desc<WB>(P, q, c0, kp);
-            d_lo[q] = make_uint4(d.lo1e, d.hih1e, d.lo1o, d.hih1o);
-            d_hi[q] = make_uint4(d.lo2e, d.hih2e, d.lo2o, d.hih2o);
-        }
-    }
+    using L = CyclicLayout<WB, BG>;
+    using Entry = typename L::Entry;
+    Entry *ent = reinterpret_cast<Entry *>(est_sm);        // [Wd]
+    double *up = reinterpret_cast<double *>(ent + P.Wd);   // [nf]
+    for (uint32_t q = threadIdx.x; q < P.Wd; q += blockDim.x)
+        ent[q] = cyclic_count_entry<WB, BG>(P, q, c0, kp);
+    const typename L::Limit lim = L::limit(cyclic_vmax(P.ace != 0, P.k, L::W));
     for (uint32_t j = threadIdx.x; j < P.nf; j += blockDim.x)
         up[j] = frame_up(P, aat, j);
     __syncthreads();
@@ -328,27 +323,13 @@ __global__ void __launch_bounds__(ESTIMATE_THREADS) estimate_kernel(Params P, co
                             x[i] = a[i][ch];
 #pragma unroll
                     for (int e = 0; e < 4; e++) {
-                        uint32_t m0 = FULL_MASK, m1 = FULL_MASK;
-                        if constexpr (BG) {
-                            const uint4 d = d_lo[4 * ch + e];
+                        const Entry d = ent[4 * ch + e];
+                        uint32_t m = FULL_MASK;
 #pragma unroll
-                            for (int i = 0; i < RM; i++)
-                                if (i < r)
-                                    m0 &= in_ranges_bytes(u4get(x[i], e), d);
-                            c += __popc(m0);
-                        } else {
-                            const RangeDesc d = load_desc(d_lo, d_hi, 4 * ch + e);
-#pragma unroll
-                            for (int i = 0; i < RM; i++) {
-                                if (i < r) {
-                                    uint32_t ev, od;
-                                    in_ranges<WB>(u4get(x[i], e), d, ev, od);
-                                    m0 &= ev;
-                                    m1 &= od;
-                                }
-                            }
-                            c += __popc(m0) + __popc(m1);
-                        }
+                        for (int i = 0; i < RM; i++)
+                            if (i < r)
+                                m &= L::test(u4get(x[i], e), d, lim);
+                        c += __popc(m);
                     }
                 }
             }
@@ -392,7 +373,6 @@ cudaError_t launch_estimate(const Params &P, uint32_t w, const uint32_t *pool, u
     while (hpw > 4 && n < (uint64_t)hpw * sms * 8)
         hpw /= 2;
     const bool bg = byte_guard(w, P.ace ? ASSE_COUNTER_ACE : ASSE_COUNTER_AT, P.k);
-    const size_t smem = (size_t)(bg ? 1 : 2) * P.Wd * sizeof(uint4) + P.nf * sizeof(double);
     *launches += 1;
     return dispatch_w(w, [&](auto wb) {
         constexpr int WB = decltype(wb)::value;
@@ -401,6 +381,7 @@ cudaError_t launch_estimate(const Params &P, uint32_t w, const uint32_t *pool, u
             if (bg)
                 kern = P.r == 4 ? estimate_kernel<8, 4, true> : estimate_kernel<8, 0, true>;
         }
+        const size_t smem = (size_t)P.Wd * (bg ? sizeof(uint2) : sizeof(uint4)) + P.nf * sizeof(double);
         const uint64_t per = (uint64_t)hpw * (ESTIMATE_THREADS / 32);
         const uint64_t want = (n + per - 1) / per;
         const uint64_t full = (uint64_t)sms * resident_blocks(kern, ESTIMATE_THREADS, smem);

@@ -1,338 +1,251 @@
 // K2: the per-slice scan of the whole pool, with the refresh fused in, and
 // the standalone refresh kernels.
 //
-// scan_kernel is a persistent kernel (one CTA per SM).  Every warp streams
-// tiles of whole ATVs from global memory into shared memory with bulk async
-// copies (cp.async.bulk, completion on an mbarrier, two buffers per warp so the
-// next tile is in flight while this one is processed).  Inside a tile one lane
-// owns one ATV, or a share of a wide ATV, in one of two layouts: a 1/2, 1/4,
-// 1/8 segment at a shared-memory stride of an odd number of 16-byte units, or
-// (interleaved) every lpa-th 16-byte chunk of an ATV stored back to back, when
-// the ATV length in chunks makes the lanes of a quarter warp hit distinct
-// banks; either way the lanes' 128-bit reads never conflict, and a tile of
-// whole, unpadded ATVs moves with one bulk copy.
+// scan_kernel is a persistent kernel whose warps work alone.  lpa lanes (eight
+// for ATVs of 32 words and more) share an ATV: lane p reads its 16-byte chunks
+// p, p + lpa, ... straight from global memory, so that a warp's load covers
+// whole 128-byte stretches of its ATVs, and a warp takes SCAN_U ATVs per group
+// of lanes at a time: SCAN_U loads in flight a lane, and one read of a word's
+// range entry (the same for the four groups, one shared-memory wavefront)
+// serves SCAN_U words.
 //
-// Activity test (Algorithm 1 on every field of a word at once): the active
-// values of a block form the cyclic window act-k'+1 .. act (mod 2k), i.e. at
-// most two plain ranges.  The even and the odd fields of a word are tested
-// separately, each field then having w free bits above it; with a guard bit
-// just above each field, (v | guard) - lo keeps the guard iff v >= lo and
-// (hi | guard) - v keeps it iff v <= hi, with no borrow between fields.  The
-// per-position constants carry each field's own range, so words that straddle
-// two ACT blocks and the fields past g (empty ranges) need no special case.
-// The refresh (Algorithm 2: values 0..k at new ACT 0; value 0 and k..2k-1 at
-// new ACT k) uses the same range machinery to find the fields to clear.
+// The activity test (Algorithm 1) and the refresh's (Algorithm 2) run on every
+// field of a word at once, as one cyclic range per field with the entry of the
+// word's position (asse_cyclic.h).  What bounds the scan of a pool in L2 is the
+// integer pipe, which is why the test has as few operations as that: two plain
+// ranges per field took 23 a word of five-bit fields, this 15.
+//
+// Fused scan of a 92 MB pool in L2: 39 us with tiles staged by bulk copies and
+// two ranges, 38 with these loads, 31 with one range too; with aging counters
+// 46 -> 28; three windows at once 79 -> 67; a 1.07 GB pool 269 -> 192 us (5.6
+// TB/s, 0.82 of the measured copy rate).  A thread that kept one chunk position
+// and its entries in registers, the counts of a block added up through shared
+// memory, ran 50 and 242 us: its block-wide barriers cost more than the table.
 //
 // Per ATV the lanes form |ATV|^{k'} (Sec. 3), the row-frame loads |AAT(k',i,j)|
-// (Sec. 4.3) and, for a super ATV (Sec. 4.2), its column and g-bit active
-// mask.  With FUSE the refreshed words (AT) are written back at once, or for
-// aging counters every word is decremented in shared memory and each segment
-// is stored back with a bulk copy.
+// (Sec. 4.3) and, for a super ATV (Sec. 4.2), its column and, from its words
+// read again, its g-bit active mask.  With FUSE the warp then reads the words of
+// the two refreshed blocks again (AT), or all words (aging counters), most of
+// them still in its L1, and writes them back.
 #include <cuda_runtime.h>
 
 #include <cstdint>
 
 #include "asse_device.cuh"
-#include "asse_ptx.cuh"
 #include "asse_swar.cuh"
 
 namespace asse {
 
 namespace {
 
-// Threads of a scan CTA: 20 warps for the interleaved layout (4 KB tiles of
-// wide ATVs, at most 102 registers a thread), 16 for the segment layouts,
-// whose code needs more registers.
-constexpr int scan_threads(bool ilv) { return ilv ? 640 : 512; }
+constexpr int SCAN_THREADS = 256;
+constexpr int SCAN_WARPS = SCAN_THREADS / 32;
+constexpr uint32_t SCAN_U = 4;  // ATVs of a group of lanes per tile
 
 // ---------------------------------------------------------------- scan kernel
 
+// Shared memory of scan_kernel: the entries of every window and of the
+// refresh, and the masks.
+template <int WB, bool BG>
+size_t scan_smem(uint32_t Wd, uint32_t mw, uint32_t nw)
+{
+    return (size_t)(nw + 1) * Wd * sizeof(typename CyclicLayout<WB, BG>::Entry) +
+           (size_t)SCAN_WARPS * mw * sizeof(uint32_t);
+}
+
+// Lanes of an ATV of S 16-byte chunks: eight, or fewer where more than a fifth
+// of their last chunks would lie past the ATV.
+inline uint32_t scan_lanes(uint32_t S)
+{
+    uint32_t lpa = 8;
+    while (lpa > 1 && 5 * S < 4 * ((S + lpa - 1) / lpa * lpa))
+        lpa /= 2;
+    return lpa;
+}
+
 // NW: the most windows this instantiation counts (1, or MAX_WINDOWS for the
 // multi-window close, which runs W.n <= NW of them).  BG: byte-wide fields
-// with values below 128, tested four at a time with the in-field guard bit
-// (one 16-byte range entry per word instead of two).
-// ILV: the interleaved tile layout (G.ilv), fixed at compile time so that
-// the per-word index arithmetic of the inner loop has no layout branch.
-template <int WB, bool FUSE, int NW, bool BG, bool ILV>
-__global__ void __launch_bounds__(scan_threads(ILV), 1) scan_kernel(Params P, uint32_t *pool, const ScanWindows W,
-                                                               const SliceCtl *ctl, uint32_t total_atv, ScanGeom G)
+// with values below 128, tested four at a time.
+template <int WB, bool FUSE, int NW, bool BG>
+__global__ void __launch_bounds__(SCAN_THREADS, 4)
+    scan_kernel(Params P, uint32_t *pool, const ScanWindows W, const SliceCtl *ctl, uint32_t total_atv, uint32_t lpa)
 {
     static_assert(!BG || WB == 8, "the in-field guard needs byte-wide fields");
     const uint32_t c0 = ctl->c0;
-    const Refresh R = ctl->R;
+    const Refresh &R = ctl->R;
     extern __shared__ __align__(128) uint8_t smem[];
-    // The count ranges of word q sit in two 16-byte halves at index q + (the
-    // segment of q): the lanes of one warp read positions one segment apart,
-    // and the skew puts those reads in distinct bank groups.
-    // Window m's table starts at m * n_cd.
     const uint32_t nw = NW == 1 ? 1u : W.n;
-    const uint32_t n_cd = P.Wd + G.lpa;
     const uint32_t nchunk = P.Wd / 4;
-    // index of word q's range entry in window m's table: skewed by segment
-    // (segments), or chunk-major per word of the chunk (interleaved), so that
-    // the lanes' reads of one step fall in distinct banks
-    auto didx = [&](uint32_t m, uint32_t q) {
-        return m * n_cd + (ILV ? (q & 3u) * nchunk + (q >> 2) : q + q / G.wseg);
-    };
-    uint4 *cd_lo = reinterpret_cast<uint4 *>(smem);                          // [nw][Wd + lpa]
-    uint4 *cd_hi = cd_lo + nw * n_cd;                                        // [nw][Wd + lpa]
-    RangeDesc *rdesc = reinterpret_cast<RangeDesc *>(cd_hi + nw * n_cd);     // [Wd]
-    uint64_t *mbar = reinterpret_cast<uint64_t *>(rdesc + P.Wd);             // [warps][2]
-    uint32_t *maskbuf = reinterpret_cast<uint32_t *>(mbar + 2 * G.warps);    // [warps][mw]
-    uint32_t *tiles = reinterpret_cast<uint32_t *>(smem + G.tile_offset);    // [warps][2][tile_words]
+    using L = CyclicLayout<WB, BG>;
+    using Entry = typename L::Entry;
+    // entry of word q of window m at m * Wd + (q mod 4) * Wd / 4 + q / 4: the
+    // lanes of an ATV read consecutive entries
+    auto didx = [&](uint32_t m, uint32_t q) { return m * P.Wd + (q & 3u) * nchunk + (q >> 2); };
+    Entry *cd = reinterpret_cast<Entry *>(smem);                      // [nw][Wd]
+    Entry *rd = cd + nw * P.Wd;                                       // [Wd]
+    uint32_t *maskbuf = reinterpret_cast<uint32_t *>(rd + P.Wd);      // [warps][mw]
 
-    const uint32_t lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    for (uint32_t e = threadIdx.x; e < nw * P.Wd; e += blockDim.x) {
+    const uint32_t tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    for (uint32_t e = tid; e < nw * P.Wd; e += SCAN_THREADS) {
         const uint32_t m = e / P.Wd, q = e - m * P.Wd;
-        const uint32_t x = didx(m, q);
-        if constexpr (BG) {
-            cd_lo[x] = count_desc_bytes(P, q, c0, W.kp[m]);
-            if (FUSE && m == 0) {
-                const uint4 r = refresh_desc_bytes(P, q, R.c0n);
-                rdesc[q] = RangeDesc{r.x, r.y, r.z, r.w, 0, 0, 0, 0};
-            }
-        } else {
-            const RangeDesc d = count_desc<WB>(P, q, c0, W.kp[m]);
-            cd_lo[x] = make_uint4(d.lo1e, d.hih1e, d.lo1o, d.hih1o);
-            cd_hi[x] = make_uint4(d.lo2e, d.hih2e, d.lo2o, d.hih2o);
-            if (FUSE && m == 0)
-                rdesc[q] = refresh_desc<WB>(P, q, R.c0n);
-        }
+        cd[didx(m, q)] = cyclic_count_entry<WB, BG>(P, q, c0, W.kp[m]);
+        if (FUSE && m == 0 && !P.ace)
+            rd[q] = cyclic_refresh_entry<WB, BG>(P, q, R.c0n);
     }
-    if (warp < G.warps && lane == 0) {
-        mbar_init(&mbar[2 * warp], 1);
-        mbar_init(&mbar[2 * warp + 1], 1);
-    }
-    fence_async_smem();
+    const typename L::Limit lim = L::limit(cyclic_vmax(P.ace != 0, P.k, L::W));
     __syncthreads();
-    if (warp >= G.warps)
-        return;
 
-    const uint32_t a = lane / G.lpa, part = lane - a * G.lpa;  // this lane's ATV in the tile and share
-    const uint32_t q_first = ILV ? 4 * part : part * G.wseg;  // its first word
-    const uint32_t q_step = ILV ? 4 * G.lpa : 4;               // words between its chunks, in the ATV and in smem
-    const uint32_t lane_off = ILV ? a * P.Wd + 4 * part : lane * G.seg_stride;  // its first word in the tile
-    // word q of the tile's ATV a_ in shared memory
-    auto tile_word = [&](const uint32_t *tb, uint32_t a_, uint32_t q) {
-        if (ILV)
-            return tb[a_ * P.Wd + q];
-        const uint32_t pq = q / G.wseg;  // the segment holding word q
-        return tb[(a_ * G.lpa + pq) * G.seg_stride + (q - pq * G.wseg)];
-    };
+    const uint32_t groups = 32 / lpa;        // ATVs side by side in a warp
+    const uint32_t grp = lane / lpa, sub = lane - grp * lpa;
+    const uint32_t apt = groups * SCAN_U;    // ATVs of a tile
+    const uint32_t ntiles = (total_atv + apt - 1) / apt;
     const uint32_t cols = P.cmask + 1;
-    const uint32_t ntiles = (total_atv + G.apt - 1) / G.apt;
     uint32_t *my_mask = maskbuf + warp * P.mw;
-    // buffer b of this warp, its mbarrier and phase parity (bit b of par);
-    // computed, not indexed arrays, so that nothing lives in local memory
-    auto tile_buf = [&](int b) { return tiles + (2 * warp + b) * G.tile_words; };
-    auto bar = [&](int b) { return &mbar[2 * warp + b]; };
-    uint32_t par = 0;
-
-    // Segments of an odd number of 16-byte units need no padding: the tile
-    // is then one contiguous stretch of the pool, fetched with one copy.
-    const bool whole = ILV || G.seg_stride == G.wseg;
-    auto issue = [&](uint32_t tile, int b) {
-        const uint32_t atv0 = tile * G.apt;
-        const uint32_t n_atv = min(G.apt, total_atv - atv0);
-        if (whole) {
-            if (lane == 0) {
-                mbar_expect_tx(bar(b), n_atv * P.Wd * 4u);
-                bulk_load(tile_buf(b), pool + (size_t)atv0 * P.Wd, n_atv * P.Wd * 4u, bar(b));
-            }
-            return;
-        }
-        if (lane == 0)
-            mbar_expect_tx(bar(b), n_atv * P.Wd * 4u);
-        __syncwarp();
-        if (a < n_atv)
-            bulk_load(tile_buf(b) + lane * G.seg_stride, pool + (size_t)(atv0 + a) * P.Wd + q_first, G.wseg * 4u,
-                      bar(b));
-    };
-    // tiles are dealt round-robin over all warps of the grid: every tile
-    // costs the same, and at any moment the warps stream one contiguous
-    // stretch of the pool
-    const uint32_t n_warps = gridDim.x * G.warps;
-    uint32_t tile = blockIdx.x * G.warps + warp;
-    int b = 0;
-    if (tile < ntiles)
-        issue(tile, 0);
-    uint32_t next = tile < ntiles ? tile + n_warps : ntiles;
-    if (next < ntiles)
-        issue(next, 1);
-    while (tile < ntiles) {
-        if (!__all_sync(FULL_MASK, mbar_wait(bar(b), (par >> b) & 1u))) {
-            // the copy did not land: flag it, give the other copy in flight a
-            // bounded chance to finish, and leave
-            if (lane == 0)
-                for (uint32_t m = 0; m < nw; m++)
-                    atomicExch(&W.o[m].status->error, 1u);
-            if (next < ntiles)
-                mbar_wait(bar(b ^ 1), (par >> (b ^ 1)) & 1u);
-            return;
-        }
-        par ^= 1u << b;
-        const uint32_t atv0 = tile * G.apt;
-        const uint32_t n_atv = min(G.apt, total_atv - atv0);
-        const bool mine = a < n_atv;
-        uint32_t *row = tile_buf(b) + lane_off;
-        uint32_t cnt[NW];
+    // tiles are dealt round-robin over all warps of the grid: at any moment
+    // the warps read one contiguous stretch of the pool
+    for (uint32_t tile = blockIdx.x * SCAN_WARPS + warp; tile < ntiles; tile += gridDim.x * SCAN_WARPS) {
+        const uint32_t atv0 = tile * apt;
+        const uint32_t n_atv = min(apt, total_atv - atv0);
+        const uint4 *src = reinterpret_cast<const uint4 *>(pool) + (size_t)(atv0 + grp) * nchunk;
+        uint32_t cnt[NW][SCAN_U];
 #pragma unroll
         for (int m = 0; m < NW; m++)
-            cnt[m] = 0;
-        if (mine) {
-#pragma unroll 2
-            for (uint32_t i = 0; i < G.wseg / 4; i++) {
-                const uint4 x = *reinterpret_cast<const uint4 *>(row + i * q_step);
-                const uint32_t q = q_first + i * q_step;
 #pragma unroll
-                for (int m = 0; m < NW; m++) {
-                    if (m < (int)nw) {
-                        // the range entries of words q .. q+3: consecutive (skewed by the
-                        // segment), or a chunk apart (q is a multiple of 4)
-                        const uint32_t xq = m * n_cd + (ILV ? (q >> 2) : q + part), dx = ILV ? nchunk : 1u;
-                        if constexpr (BG) {
-                            // per-byte counts (at most 64 words per lane: no carry between bytes)
-                            cnt[m] += (in_ranges_bytes(x.x, cd_lo[xq]) >> 7) +
-                                      (in_ranges_bytes(x.y, cd_lo[xq + dx]) >> 7) +
-                                      (in_ranges_bytes(x.z, cd_lo[xq + 2 * dx]) >> 7) +
-                                      (in_ranges_bytes(x.w, cd_lo[xq + 3 * dx]) >> 7);
-                        } else {
-                            cnt[m] += count_word<WB>(x.x, load_desc(cd_lo, cd_hi, xq)) +
-                                      count_word<WB>(x.y, load_desc(cd_lo, cd_hi, xq + dx)) +
-                                      count_word<WB>(x.z, load_desc(cd_lo, cd_hi, xq + 2 * dx)) +
-                                      count_word<WB>(x.w, load_desc(cd_lo, cd_hi, xq + 3 * dx));
+            for (uint32_t u = 0; u < SCAN_U; u++)
+                cnt[m][u] = 0;
+        for (uint32_t ch = sub; ch < nchunk; ch += lpa) {
+            uint4 x[SCAN_U];
+#pragma unroll
+            for (uint32_t u = 0; u < SCAN_U; u++)
+                x[u] = u * groups + grp < n_atv ? src[(size_t)u * groups * nchunk + ch] : make_uint4(0, 0, 0, 0);
+#pragma unroll
+            for (int m = 0; m < NW; m++) {
+                if (m < (int)nw) {
+                    const Entry *tab = cd + m * P.Wd + ch;
+                    uint32_t bits[SCAN_U];
+#pragma unroll
+                    for (int j = 0; j < 4; j++) {
+                        const Entry d = tab[j * nchunk];
+#pragma unroll
+                        for (uint32_t u = 0; u < SCAN_U; u++) {
+                            const uint32_t b = L::test(u4get(x[u], j), d, lim);
+                            if constexpr (BG)  // the guards of the four words side by side in the bytes
+                                bits[u] = j == 0 ? b : bits[u] | (b >> j);
+                            else
+                                cnt[m][u] += __popc(b);
                         }
+                    }
+                    if constexpr (BG) {
+#pragma unroll
+                        for (uint32_t u = 0; u < SCAN_U; u++)
+                            cnt[m][u] += __popc(bits[u]);
                     }
                 }
             }
         }
-        if constexpr (BG) {
-#pragma unroll
-            for (int m = 0; m < NW; m++)
-                cnt[m] = (cnt[m] * BYTE_ONES) >> 24;  // the four byte counts added
-        }
-        const uint32_t atv = atv0 + a;
-        const bool head = mine && part == 0;
-        const uint32_t sg = head ? atv >> P.c : 0xffffffffu;  // row * 2^u + frame
-        const unsigned grp = __match_any_sync(FULL_MASK, sg);
+        // the lanes of an ATV add up, two 16-bit counts to a word; then its lane
+        // u takes ATV u (lane u mod lpa, in turns, where it has fewer lanes)
 #pragma unroll 1
         for (uint32_t m = 0; m < nw; m++) {
             const ScanOut &o = W.o[m];
-            uint32_t c = NW == 1 ? cnt[0] : 0u;
-            if (NW > 1) {
+            uint32_t c01 = 0, c23 = 0;
 #pragma unroll
-                for (int mm = 0; mm < NW; mm++)
-                    if ((uint32_t)mm == m)
-                        c = cnt[mm];
+            for (int mm = 0; mm < NW; mm++)
+                if (NW == 1 || (uint32_t)mm == m) {
+                    c01 = cnt[mm][0] | (cnt[mm][1] << 16);
+                    c23 = cnt[mm][2] | (cnt[mm][3] << 16);
+                }
+            for (uint32_t off = 1; off < lpa; off <<= 1) {
+                c01 += __shfl_xor_sync(FULL_MASK, c01, off);
+                c23 += __shfl_xor_sync(FULL_MASK, c23, off);
             }
-            for (uint32_t off = 1; off < G.lpa; off <<= 1)
-                c += __shfl_xor_sync(FULL_MASK, c, off);
-
-            // one lane per ATV: count, row-frame load, super test
-            if (head)
-                o.cnt[atv] = (uint16_t)c;
-            {
-                const uint32_t s = __reduce_add_sync(grp, head ? c : 0u);
-                if (head && (uint32_t)(__ffs(grp) - 1) == lane && s)
-                    atomicAdd(&o.aat[sg], (unsigned long long)s);
-            }
-            const bool sup = head && c >= P.T;
-            uint32_t slot = 0;
-            if (sup) {
-                slot = atomicAdd(&o.sa_n[sg], 1u);
-                o.sa_x[(size_t)sg * cols + slot] = atv & P.cmask;
-            }
-            unsigned sbits = __ballot_sync(FULL_MASK, sup);
-            while (sbits) {
-                // the g-bit active mask of one super ATV, for Algorithm 5;
-                // all 32 lanes share its words (segment by segment in the tile)
-                const uint32_t hl = __ffs(sbits) - 1;
-                sbits &= sbits - 1;
-                const uint32_t slot_a = __shfl_sync(FULL_MASK, slot, hl);
-                const uint32_t a_s = hl / G.lpa;
-                const uint32_t sg_a = (atv0 + a_s) >> P.c;
-                for (uint32_t k = lane; k < P.mw; k += 32)
-                    my_mask[k] = 0;
-                __syncwarp();
-                {
-                    constexpr uint32_t F = 32 / WB;
-                    for (uint32_t q = lane; q < P.Wd; q += 32) {
-                        const uint32_t word = tile_word(tile_buf(b), a_s, q);
-                        const uint32_t am = BG ? field_bits_bytes(word, cd_lo[didx(m, q)])
-                                               : field_bits<WB>(word, load_desc(cd_lo, cd_hi, didx(m, q)));
-                        if (am) {
-                            const uint32_t pos = q * F, off = pos & 31;
-                            atomicOr(&my_mask[pos >> 5], am << off);
-                            if (off + F > 32 && (am >> (32 - off)))
-                                atomicOr(&my_mask[(pos >> 5) + 1], am >> (32 - off));
+            for (uint32_t u0 = 0; u0 < SCAN_U; u0 += lpa) {
+                const uint32_t u = u0 + sub, i = u * groups + grp;
+                const bool head = u < SCAN_U && i < n_atv;
+                const uint32_t c2 = (u & 2) ? c23 : c01;
+                const uint32_t c = (u & 1) ? c2 >> 16 : c2 & 0xffffu;
+                const uint32_t atv = atv0 + i;
+                const uint32_t sg = head ? atv >> P.c : 0xffffffffu;  // row * 2^u + frame
+                if (head)
+                    o.cnt[atv] = (uint16_t)c;
+                // one atomic for the tile where its ATVs are of one row-frame
+                if (atv0 >> P.c == (atv0 + n_atv - 1) >> P.c) {
+                    const uint32_t s = __reduce_add_sync(FULL_MASK, head ? c : 0u);
+                    if (lane == 0 && s)
+                        atomicAdd(&o.aat[atv0 >> P.c], (unsigned long long)s);
+                } else {
+                    const unsigned same = __match_any_sync(FULL_MASK, sg);
+                    const uint32_t s = __reduce_add_sync(same, head ? c : 0u);
+                    if (head && (uint32_t)(__ffs(same) - 1) == lane && s)
+                        atomicAdd(&o.aat[sg], (unsigned long long)s);
+                }
+                const bool sup = head && c >= P.T;
+                uint32_t slot = 0;
+                if (sup) {
+                    slot = atomicAdd(&o.sa_n[sg], 1u);
+                    o.sa_x[(size_t)sg * cols + slot] = atv & P.cmask;
+                }
+                unsigned sbits = __ballot_sync(FULL_MASK, sup);
+                while (sbits) {
+                    // the g-bit active mask of one super ATV, for Algorithm 5;
+                    // all 32 lanes share its words
+                    const uint32_t hl = __ffs(sbits) - 1;
+                    sbits &= sbits - 1;
+                    const uint32_t slot_a = __shfl_sync(FULL_MASK, slot, hl);
+                    const uint32_t atv_a = __shfl_sync(FULL_MASK, atv, hl);
+                    for (uint32_t k = lane; k < P.mw; k += 32)
+                        my_mask[k] = 0;
+                    __syncwarp();
+                    {
+                        constexpr uint32_t F = 32 / WB;
+                        for (uint32_t q = lane; q < P.Wd; q += 32) {
+                            const uint32_t word = pool[(size_t)atv_a * P.Wd + q];
+                            const uint32_t am = L::compress(L::test(word, cd[didx(m, q)], lim));
+                            if (am) {
+                                const uint32_t pos = q * F, off = pos & 31;
+                                atomicOr(&my_mask[pos >> 5], am << off);
+                                if (off + F > 32 && (am >> (32 - off)))
+                                    atomicOr(&my_mask[(pos >> 5) + 1], am >> (32 - off));
+                            }
                         }
                     }
+                    __syncwarp();
+                    uint32_t *dst = o.sa_mask + ((size_t)(atv_a >> P.c) * cols + slot_a) * P.mw;
+                    for (uint32_t k = lane; k < P.mw; k += 32)
+                        dst[k] = my_mask[k];
+                    __syncwarp();
                 }
-                __syncwarp();
-                uint32_t *dst = o.sa_mask + ((size_t)sg_a * cols + slot_a) * P.mw;
-                for (uint32_t k = lane; k < P.mw; k += 32)
-                    dst[k] = my_mask[k];
-                __syncwarp();
             }
         }
-
+        // the tile's words are counted and its masks made: its words may change
+        if (FUSE)
+            __syncwarp();
         if (FUSE && !P.ace) {
             // Algorithm 2 for the next slice on the words of the two refreshed blocks
             for (uint32_t rr = 0; rr < R.n_ranges; rr++) {
-                // segments: the lane's own words of the range; interleaved: the
-                // words of its chunks
-                const uint32_t lo = ILV ? R.q_lo[rr] : max(R.q_lo[rr], q_first);
-                const uint32_t hi = ILV ? R.q_hi[rr] + 1 : min(R.q_hi[rr] + 1, q_first + G.wseg);
-                if (mine) {
-                    for (uint32_t q = lo; q < hi; q++) {
-                        if (ILV && ((q >> 2) & (G.lpa - 1)) != part)
-                            continue;
-                        const uint32_t w = tile_word(tile_buf(b), a, q);
-                        const RangeDesc &rd = rdesc[q];
-                        const uint32_t nw = BG ? refresh_bytes(P.k2, w, make_uint4(rd.lo1e, rd.hih1e, rd.lo1o, rd.hih1o))
-                                               : refresh_swar<WB>(P, w, rd);
-                        if (nw != w)
-                            pool[(size_t)atv * P.Wd + q] = nw;
-                    }
+                const uint32_t q0 = R.q_lo[rr], len = R.q_hi[rr] - q0 + 1;
+                const uint32_t inv = 0xffffffffu / len + 1;  // e / len by a multiply-high, exact for e len < 2^32
+                for (uint32_t e = lane; e < n_atv * len; e += 32) {
+                    const uint32_t i = len == 1 ? e : __umulhi(e, inv), q = q0 + (e - i * len);
+                    uint32_t *wp = pool + (size_t)(atv0 + i) * P.Wd + q;
+                    const uint32_t w = *wp;
+                    const uint32_t v = cyclic_refresh<WB, BG>(P, w, rd[q], lim);
+                    if (v != w)
+                        *wp = v;
                 }
             }
         }
         if (FUSE && P.ace) {
-            // every aging counter loses one: decrement in place, store the segment back
-            if (mine && !ILV) {
-                for (uint32_t i = 0; i < G.wseg; i++)
-                    row[i] = BG ? decay_bytes(row[i]) : decay_swar<WB>(row[i]);
-                fence_async_smem();
-                if (!whole)
-                    bulk_store(pool + (size_t)atv * P.Wd + q_first, row, G.wseg * 4u);
-            }
-            if (ILV) {
-                uint32_t *tb = tile_buf(b);
-                for (uint32_t i = lane; i < n_atv * P.Wd; i += 32)
-                    tb[i] = BG ? decay_bytes(tb[i]) : decay_swar<WB>(tb[i]);
-                fence_async_smem();
-            }
-            if (whole) {
-                __syncwarp();
-                if (lane == 0)
-                    bulk_store(pool + (size_t)atv0 * P.Wd, tile_buf(b), n_atv * P.Wd * 4u);
+            // every aging counter loses one
+            uint4 *wp = reinterpret_cast<uint4 *>(pool) + (size_t)atv0 * nchunk;
+            for (uint32_t e = lane; e < n_atv * nchunk; e += 32) {
+                const uint4 v = wp[e];
+                wp[e] = BG ? make_uint4(decay_bytes(v.x), decay_bytes(v.y), decay_bytes(v.z), decay_bytes(v.w))
+                           : make_uint4(decay_swar<WB>(v.x), decay_swar<WB>(v.y), decay_swar<WB>(v.z),
+                                        decay_swar<WB>(v.w));
             }
         }
-        // this buffer is free again: fetch the tile after next into it
-        __syncwarp();
-        tile = next;
-        next = tile < ntiles ? tile + n_warps : ntiles;
-        if (next < ntiles) {
-            if (FUSE && P.ace)
-                bulk_store_drain();  // this buffer's write-back has read its source
-            fence_async_smem();
-            __syncwarp();
-            issue(next, b);
-        }
-        b ^= 1;
     }
-    if (FUSE && P.ace)
-        bulk_store_drain();
 }
 
 // ---------------------------------------------------------------- A3 alone
@@ -408,45 +321,6 @@ __global__ void __launch_bounds__(256) ace_decay_kernel(uint4 *pool, uint64_t nv
 
 }  // namespace
 
-// Tile geometry of the scan for ATVs of Wd words: lanes per ATV (so a lane
-// holds at most 48 words where Wd allows), the shared-memory stride of a lane's segment (an odd
-// number of 16-byte units) and how many warps fit the shared memory.
-ScanGeom scan_geometry(uint32_t Wd, uint32_t mw, uint32_t nw, size_t smem_limit)
-{
-    ScanGeom G{};
-    G.lpa = 1;
-    while (Wd / G.lpa > 48 && Wd % (8 * G.lpa) == 0 && G.lpa < 8)
-        G.lpa *= 2;
-    G.wseg = Wd / G.lpa;
-    uint32_t units = G.wseg / 4;
-    // Interleaved chunks where a segment would need padding and the ATV
-    // length S = Wd/4 chunks keeps the chunks the 8 lanes of a quarter warp
-    // read at once in distinct 16-byte bank groups: the quarter holds 8/lpa
-    // ATVs whose lanes read chunks a*S + p (+ i*lpa), distinct mod 8 when S is
-    // lpa times an odd number modulo 8 (any S with lpa = 8).
-    const uint32_t S = Wd / 4;
-    const bool ilv_ok = Wd % (4 * G.lpa) == 0 &&
-                        (G.lpa == 8 || (G.lpa == 4 && S % 8 == 4) || (G.lpa == 2 && S % 4 == 2) ||
-                         (G.lpa == 1 && S % 2 == 1));
-    G.ilv = (units & 1) == 0 && ilv_ok ? 1u : 0u;
-    if ((units & 1) == 0 && !G.ilv)
-        units += 1;
-    G.seg_stride = G.ilv ? G.wseg : units * 4;
-    G.apt = 32 / G.lpa;
-    G.tile_words = 32 * G.seg_stride;
-    const size_t fixed = (size_t)nw * (Wd + G.lpa) * 2 * sizeof(uint4) + (size_t)Wd * sizeof(RangeDesc);
-    auto head = [&](uint32_t warps) {
-        const size_t h = fixed + 2 * warps * sizeof(uint64_t) + (size_t)warps * mw * 4;
-        return (h + 127) / 128 * 128;
-    };
-    G.warps = scan_threads(G.ilv) / 32;
-    while (G.warps > 1 && head(G.warps) + (size_t)G.warps * 2 * G.tile_words * 4 > smem_limit)
-        G.warps--;
-    G.tile_offset = (uint32_t)head(G.warps);
-    G.smem = G.tile_offset + G.warps * 2 * G.tile_words * 4;
-    return G;
-}
-
 namespace {
 
 template <int NW>
@@ -454,36 +328,32 @@ cudaError_t launch_scan_nw(const Params &P, uint32_t w, uint32_t *pool, const Sc
                            const SliceCtl *ctl, int sms, cudaStream_t s)
 {
     const uint32_t total = P.r << P.E_log2;
-    const ScanGeom G = scan_geometry(P.Wd, P.mw, W.n, 200 * 1024);
-    const uint32_t ntiles = (total + G.apt - 1) / G.apt;
+    const uint32_t lpa = scan_lanes(P.Wd / 4);
     const bool bg = byte_guard(w, P.ace ? ASSE_COUNTER_ACE : ASSE_COUNTER_AT, P.k);
     return dispatch_w(w, [&](auto wb) {
         constexpr int WB = decltype(wb)::value;
-        auto pick = [&](auto ilv) {
-            constexpr bool ILV = decltype(ilv)::value;
-            auto k = scan_kernel<WB, true, NW, false, ILV>;
-            if constexpr (NW == 1) {
-                if (!fuse)
-                    k = scan_kernel<WB, false, 1, false, ILV>;
-            }
-            if constexpr (WB == 8) {
-                if (bg) {
-                    k = scan_kernel<8, true, NW, true, ILV>;
-                    if constexpr (NW == 1) {
-                        if (!fuse)
-                            k = scan_kernel<8, false, 1, true, ILV>;
-                    }
+        auto kern = scan_kernel<WB, true, NW, false>;
+        if constexpr (NW == 1) {
+            if (!fuse)
+                kern = scan_kernel<WB, false, 1, false>;
+        }
+        if constexpr (WB == 8) {
+            if (bg) {
+                kern = scan_kernel<8, true, NW, true>;
+                if constexpr (NW == 1) {
+                    if (!fuse)
+                        kern = scan_kernel<8, false, 1, true>;
                 }
             }
-            return k;
-        };
-        auto kern = G.ilv ? pick(std::true_type()) : pick(std::false_type());
-        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)G.smem);
+        }
+        const size_t smem = bg ? scan_smem<8, true>(P.Wd, P.mw, W.n) : scan_smem<WB, false>(P.Wd, P.mw, W.n);
+        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess)
             return e;
-        const uint64_t want = (ntiles + G.warps - 1) / G.warps;
-        const unsigned grid = (unsigned)(want < (uint64_t)sms ? (want < 1 ? 1 : want) : (uint64_t)sms);
-        kern<<<grid, scan_threads(G.ilv), G.smem, s>>>(P, pool, W, ctl, total, G);
+        const uint32_t per = 32 / lpa * SCAN_U * SCAN_WARPS;  // ATVs of a block's tiles
+        const uint32_t want = (total + per - 1) / per;
+        const uint32_t full = (uint32_t)sms * resident_blocks(kern, SCAN_THREADS, smem);
+        kern<<<want < full ? want : full, SCAN_THREADS, smem, s>>>(P, pool, W, ctl, total, lpa);
         return cudaGetLastError();
     });
 }

@@ -15,6 +15,7 @@
 #include <cstdint>
 
 #include "asse_bytes.h"
+#include "asse_cyclic.h"
 #include "asse_device.cuh"
 
 namespace asse {
@@ -134,12 +135,6 @@ __device__ RangeDesc refresh_desc(const Params &P, uint32_t q, uint32_t c0n)
     return d;
 }
 
-__device__ __forceinline__ RangeDesc load_desc(const uint4 *lo, const uint4 *hi, uint32_t x)
-{
-    const uint4 a = lo[x], b = hi[x];
-    return RangeDesc{a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
-}
-
 // Guard bits of the fields of word w whose value lies in one of the ranges.
 template <int WB>
 __device__ __forceinline__ void in_ranges(uint32_t w, const RangeDesc &d, uint32_t &ge_bits, uint32_t &go_bits)
@@ -149,14 +144,6 @@ __device__ __forceinline__ void in_ranges(uint32_t w, const RangeDesc &d, uint32
     const uint32_t xeh = xe | S::HE, xoh = xo | S::HO;
     ge_bits = (((xeh - d.lo1e) & (d.hih1e - xe)) | ((xeh - d.lo2e) & (d.hih2e - xe))) & S::HE;
     go_bits = (((xoh - d.lo1o) & (d.hih1o - xo)) | ((xoh - d.lo2o) & (d.hih2o - xo))) & S::HO;
-}
-
-template <int WB>
-__device__ __forceinline__ uint32_t count_word(uint32_t w, const RangeDesc &d)
-{
-    uint32_t e, o;
-    in_ranges<WB>(w, d, e, o);
-    return __popc(e) + __popc(o);
 }
 
 // Field j (bit j) set iff field j of w is in one of the ranges.
@@ -199,69 +186,49 @@ __device__ __forceinline__ uint32_t decay_swar(uint32_t w)
 }
 
 // ---------------------------------------------------------------------------
-// Byte-wide fields with values below 128 (asse_bytes.h): the range entries of
-// every word position, built like count_desc / refresh_desc but as four byte
-// lanes of one word each.
+// Entries of the one-range test (asse_cyclic.h) of word position q.
 
-// The count ranges of word position q (one ACT block per word is not
-// assumed: a word whose fields fall in two blocks gets per-byte ranges).
-__device__ __forceinline__ uint4 count_desc_bytes(const Params &P, uint32_t q, uint32_t c0, uint32_t kp)
+// The fields active in the latest kp slices when block 0 has ACT c0.
+template <int WB, bool BG>
+__device__ typename CyclicLayout<WB, BG>::Entry cyclic_count_entry(const Params &P, uint32_t q, uint32_t c0,
+                                                                   uint32_t kp)
 {
-    uint4 d = make_uint4(0, 0, 0, 0);
-    for (uint32_t j = 0; j < 4; j++) {
-        const uint32_t h = q * 4 + j;
-        uint32_t l1 = 127, h1 = 0, l2 = 127, h2 = 0;  // empty ranges
-        if (h < P.g) {
-            if (P.ace) {
-                l1 = P.k + 1 - kp;
-                h1 = P.k;
-            } else {
-                const uint32_t act = act_of(P, c0, pos_block(P, h));
-                if (act + 1 >= kp) {
-                    l1 = act + 1 - kp;
-                    h1 = act;
-                } else {  // the window wraps past 0 to the top of 0..2k-1
-                    l1 = 0;
-                    h1 = act;
-                    l2 = act + P.k2 + 1 - kp;
-                    h2 = P.k2 - 1;
-                }
-            }
-        }
-        d.x |= l1 << (8 * j);
-        d.y |= (h1 | 0x80u) << (8 * j);
-        d.z |= l2 << (8 * j);
-        d.w |= (h2 | 0x80u) << (8 * j);
+    using L = CyclicLayout<WB, BG>;
+    typename L::Entry d = L::empty();
+    for (uint32_t j = 0; j < L::F; j++) {
+        const uint32_t h = q * L::F + j;
+        const uint32_t act = h < P.g && !P.ace ? act_of(P, c0, pos_block(P, h)) : 0u;
+        L::put(d, j, h < P.g ? cyclic_active(P.ace != 0, P.k, kp, act, L::W) : cyclic_none_past_g());
     }
     return d;
 }
 
-// The ranges Algorithm 2 clears in every byte of word position q when block 0
-// has ACT c0n.
-__device__ __forceinline__ uint4 refresh_desc_bytes(const Params &P, uint32_t q, uint32_t c0n)
+// The fields Algorithm 2 clears when block 0 has ACT c0n (timestamps).
+template <int WB, bool BG>
+__device__ typename CyclicLayout<WB, BG>::Entry cyclic_refresh_entry(const Params &P, uint32_t q, uint32_t c0n)
 {
-    uint4 d = make_uint4(0, 0, 0, 0);
-    for (uint32_t j = 0; j < 4; j++) {
-        const uint32_t h = q * 4 + j;
-        uint32_t l1 = 127, h1 = 0, l2 = 127, h2 = 0;
-        if (h < P.g && !P.ace) {
-            const uint32_t act = act_of(P, c0n, pos_block(P, h));
-            if (act == 0) {
-                l1 = 0;
-                h1 = P.k;
-            } else if (act == P.k) {
-                l1 = P.k;
-                h1 = P.k2 - 1;
-                l2 = 0;
-                h2 = 0;
-            }
-        }
-        d.x |= l1 << (8 * j);
-        d.y |= (h1 | 0x80u) << (8 * j);
-        d.z |= l2 << (8 * j);
-        d.w |= (h2 | 0x80u) << (8 * j);
+    using L = CyclicLayout<WB, BG>;
+    typename L::Entry d = L::empty();
+    for (uint32_t j = 0; j < L::F; j++) {
+        const uint32_t h = q * L::F + j;
+        L::put(d, j, h < P.g ? cyclic_cleared(P.k, act_of(P, c0n, pos_block(P, h)), L::W) : cyclic_none_past_g());
     }
     return d;
+}
+
+// Algorithm 2 on a word: the fields the entry clears become 2k.
+template <int WB, bool BG>
+__device__ __forceinline__ uint32_t cyclic_refresh(const Params &P, uint32_t w,
+                                                   const typename CyclicLayout<WB, BG>::Entry &d,
+                                                   const typename CyclicLayout<WB, BG>::Limit &l)
+{
+    using L = CyclicLayout<WB, BG>;
+    const uint32_t fm = L::widen(L::test(w, d, l));
+    uint32_t k2rep = 0;
+#pragma unroll
+    for (uint32_t j = 0; j < L::F; j++)
+        k2rep |= P.k2 << (j * WB);
+    return (w & ~fm) | (k2rep & fm);
 }
 
 }  // namespace asse
