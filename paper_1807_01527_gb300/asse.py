@@ -560,14 +560,14 @@ class MLP:
 
     def backward(self, x, t):
         import torch
-        loss = torch.zeros(1, dtype=torch.float32, device=x.device)
+        loss = torch.empty(1, dtype=torch.float32, device=x.device)  # written by the call
         self._check(lib().asse_mlp_backward(self._h, vp(x.data_ptr()), vp(t.data_ptr()), x.shape[0],
                                             vp(loss.data_ptr())))
         return loss
 
     def train_step(self, x, t, lr: float):
         import torch
-        loss = torch.zeros(1, dtype=torch.float32, device=x.device)
+        loss = torch.empty(1, dtype=torch.float32, device=x.device)  # written by the call
         self._check(lib().asse_mlp_train_step(self._h, vp(x.data_ptr()), vp(t.data_ptr()), x.shape[0], lr,
                                               vp(loss.data_ptr())))
         return loss

@@ -7,10 +7,10 @@
 // one kernel whose operands are addressed by (row, k) strides
 // (launch_tc_gemm, asse_mlp_tc.cu), so the forward products and the
 // transposed ones of the weight gradients (split over the batch) are the same
-// kernel with a different epilogue: bias + ReLU -> BF16, bias + ReLU + dot
-// with w3 (the last layer fused into the second), gradient masked by the
-// ReLU -> BF16, or FP32 atomic accumulation.  Inference has its own fused
-// tcgen05 kernel.
+// kernel with a different epilogue: bias + ReLU -> BF16, the same + dot with w3
+// (the last layer fused into the second), gradient masked by the ReLU -> BF16
+// with its column sums, or FP32 atomic accumulation.  A step is six launches.
+// Inference has its own fused tcgen05 kernel.
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
@@ -263,75 +263,114 @@ __global__ void __launch_bounds__(SYNTH_WARPS * 32) synth_kernel(Params P, Synth
 
 // ---------------------------------------------------------------- elementwise
 
-__global__ void fill_kernel(float *y, uint64_t n, const float *value)
-{
-    for (uint64_t i = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; i < n; i += (uint64_t)gridDim.x * blockDim.x)
-        y[i] = *value;
-}
-
-// Squared error of the log: dy = 2 (y - t) / n, loss += (y - t)^2 / n.
+// From the eight partial sums of every output (columns 32 q .. of the second
+// layer, q = 0..7; y = b3 + their sum) to the gradient of the second layer's
+// outputs.  Squared error of the log: dy = 2 (y - t) / n, loss += (y - t)^2 / n.
 // Squared relative error of the estimate exp(y) against exp(t): with
 // e = exp(y - t), loss += (e - 1)^2 / n and dy = 2 (e - 1) e / n (y - t
-// clamped at 20 so that e stays finite).
-__global__ void loss_kernel(const float *y, const float *t, uint64_t n, int kind, float *dy, float *loss)
+// clamped at 20 so that e stays finite).  Then dZ2 = bf16(dy[m] w3[n] [H2 > 0]);
+// dw3[n] += dy[m] H2[m][n]; db2[n] += dZ2; db3 += dy.
+//
+// A block takes 32 rows at a time: a lane of its first warp per row for dy, then
+// a warp per row, a lane per eight columns (16-byte loads and stores).  The sums
+// stay in registers until the block's last row, so that a column takes one
+// atomic per block (n / 32 of them; with 2,048 blocks of a thread per column
+// they were most of 18 us, 4,096 rows).
+constexpr int OUT_ROWS = 32;
+__global__ void __launch_bounds__(256) out_grad_kernel(const float *yp, const float *b3, const float *t, uint64_t n,
+                                                       int kind, const bf16 *H2, const float *w3, bf16 *dZ2,
+                                                       float *g_w3, float *g_b2, float *g_b3, float *loss)
 {
-    float acc = 0.0f;
-    for (uint64_t i = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; i < n; i += (uint64_t)gridDim.x * blockDim.x) {
-        const float d = y[i] - t[i];
-        if (kind == ASSE_LOSS_REL_MSE) {
-            const float e = expf(fminf(d, 20.0f));
-            dy[i] = 2.0f * (e - 1.0f) * e / (float)n;
-            acc += (e - 1.0f) * (e - 1.0f) / (float)n;
-        } else {
-            dy[i] = 2.0f * d / (float)n;
-            acc += d * d / (float)n;
+    __shared__ float dy[OUT_ROWS];
+    __shared__ float red[8][2][HID];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    float w[8], sw[8], sb[8], s3 = 0.0f, sl = 0.0f;
+#pragma unroll
+    for (int i = 0; i < 8; i++) {
+        w[i] = w3[lane * 8 + i];
+        sw[i] = sb[i] = 0.0f;
+    }
+    for (uint64_t base = (uint64_t)blockIdx.x * OUT_ROWS; base < n; base += (uint64_t)gridDim.x * OUT_ROWS) {
+        __syncthreads();  // the last rows' dy are read
+        if (warp == 0) {
+            const uint64_t m = base + lane;
+            float g = 0.0f;
+            if (m < n) {
+                float y = *b3;
+#pragma unroll
+                for (int q = 0; q < HID / 32; q++)
+                    y += yp[q * n + m];
+                const float d = y - t[m];
+                if (kind == ASSE_LOSS_REL_MSE) {
+                    const float e = expf(fminf(d, 20.0f));
+                    g = 2.0f * (e - 1.0f) * e / (float)n;
+                    sl += (e - 1.0f) * (e - 1.0f) / (float)n;
+                } else {
+                    g = 2.0f * d / (float)n;
+                    sl += d * d / (float)n;
+                }
+                s3 += g;
+            }
+            dy[lane] = g;
+        }
+        __syncthreads();
+#pragma unroll
+        for (int rr = 0; rr < OUT_ROWS; rr += 8) {
+            const uint64_t m = base + rr + warp;
+            if (m >= n)
+                break;
+            const float d = dy[rr + warp];
+            const uint4 h4 = *reinterpret_cast<const uint4 *>(H2 + m * HID + lane * 8);
+            uint32_t z4[4];
+#pragma unroll
+            for (int i = 0; i < 4; i++) {
+                const uint32_t hw = u4get(h4, i);
+                uint32_t zz = 0;
+#pragma unroll
+                for (int b = 0; b < 2; b++) {
+                    const int c = 2 * i + b;
+                    const float h = __uint_as_float(b ? hw & 0xffff0000u : hw << 16);
+                    const bf16 z = __float2bfloat16_rn(h > 0.0f ? d * w[c] : 0.0f);
+                    zz |= (uint32_t)__bfloat16_as_ushort(z) << (16 * b);
+                    sw[c] += d * h;
+                    sb[c] += __bfloat162float(z);
+                }
+                z4[i] = zz;
+            }
+            *reinterpret_cast<uint4 *>(dZ2 + m * HID + lane * 8) = make_uint4(z4[0], z4[1], z4[2], z4[3]);
         }
     }
-    acc += __shfl_xor_sync(FULL_MASK, acc, 16);
-    acc += __shfl_xor_sync(FULL_MASK, acc, 8);
-    acc += __shfl_xor_sync(FULL_MASK, acc, 4);
-    acc += __shfl_xor_sync(FULL_MASK, acc, 2);
-    acc += __shfl_xor_sync(FULL_MASK, acc, 1);
-    if ((threadIdx.x & 31) == 0)
-        atomicAdd(loss, acc);
-}
-
-// dZ2 = bf16(dy[m] w3[n] [H2 > 0]); dw3[n] += dy[m] H2[m][n]; db2[n] += dZ2;
-// db3 += dy.  One block of HID threads per chunk of rows.
-__global__ void __launch_bounds__(HID) out_grad_kernel(const float *dy, const bf16 *H2, const float *w3, uint64_t n,
-                                                       bf16 *dZ2, float *g_w3, float *g_b2, float *g_b3)
-{
-    const int col = threadIdx.x;
-    float sw = 0.0f, sb = 0.0f, s3 = 0.0f;
-    for (uint64_t m = blockIdx.x; m < n; m += gridDim.x) {
-        const float d = dy[m];
-        const float h = __bfloat162float(H2[m * HID + col]);
-        const bf16 z = __float2bfloat16_rn(h > 0.0f ? d * w3[col] : 0.0f);
-        dZ2[m * HID + col] = z;
-        sw += d * h;
-        sb += __bfloat162float(z);
-        if (col == 0)
-            s3 += d;
+#pragma unroll
+    for (int i = 0; i < 8; i++) {
+        red[warp][0][lane * 8 + i] = sw[i];
+        red[warp][1][lane * 8 + i] = sb[i];
     }
-    atomicAdd(&g_w3[col], sw);
-    atomicAdd(&g_b2[col], sb);
-    if (col == 0)
-        atomicAdd(g_b3, s3);
+    __syncthreads();
+    float a = 0.0f, b = 0.0f;
+#pragma unroll
+    for (int v = 0; v < 8; v++) {
+        a += red[v][0][threadIdx.x];
+        b += red[v][1][threadIdx.x];
+    }
+    atomicAdd(&g_w3[threadIdx.x], a);
+    atomicAdd(&g_b2[threadIdx.x], b);
+    if (warp == 0) {
+#pragma unroll
+        for (int off = 16; off >= 1; off >>= 1) {
+            s3 += __shfl_xor_sync(FULL_MASK, s3, off);
+            sl += __shfl_xor_sync(FULL_MASK, sl, off);
+        }
+        if (lane == 0) {
+            atomicAdd(g_b3, s3);
+            atomicAdd(loss, sl);
+        }
+    }
 }
 
-// g_b[n] += sum over rows of Z[m][n]
-__global__ void __launch_bounds__(HID) colsum_kernel(const bf16 *Z, uint64_t n, float *g_b)
-{
-    const int col = threadIdx.x;
-    float s = 0.0f;
-    for (uint64_t m = blockIdx.x; m < n; m += gridDim.x)
-        s += __bfloat162float(Z[m * HID + col]);
-    atomicAdd(&g_b[col], s);
-}
-
-// Adam on the fp32 parameters, refreshing the bf16 copies of W1 and W2.
+// Adam on the fp32 parameters, refreshing the bf16 copies of W1 and W2, as
+// they are and packed for the inference kernel.
 __global__ void adam_kernel(float *p, const float *gr, float *m1, float *m2, uint64_t n, float lr, float b1t,
-                            float b2t, bf16 *w1b, bf16 *w2b)
+                            float b2t, bf16 *w1b, bf16 *w2b, bf16 *w1p, bf16 *w2p)
 {
     for (uint64_t i = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; i < n; i += (uint64_t)gridDim.x * blockDim.x) {
         const float g = gr[i];
@@ -341,10 +380,13 @@ __global__ void adam_kernel(float *p, const float *gr, float *m1, float *m2, uin
         m2[i] = b;
         const float v = p[i] - lr * (a / b1t) / (sqrtf(b / b2t) + 1e-8f);
         p[i] = v;
-        if (i < OFF_B1)
-            w1b[i - OFF_W1] = __float2bfloat16_rn(v);
-        else if (i >= OFF_W2 && i < OFF_B2)
-            w2b[i - OFF_W2] = __float2bfloat16_rn(v);
+        if (i < OFF_B1) {
+            const uint32_t e = (uint32_t)(i - OFF_W1);
+            w1p[mlp_w1p_at(e / FEAT, e % FEAT)] = w1b[e] = __float2bfloat16_rn(v);
+        } else if (i >= OFF_W2 && i < OFF_B2) {
+            const uint32_t e = (uint32_t)(i - OFF_W2);
+            w2p[mlp_w2p_at(e / HID, e % HID)] = w2b[e] = __float2bfloat16_rn(v);
+        }
     }
 }
 
@@ -373,7 +415,8 @@ struct asse_mlp {
     int *error = nullptr;                 // set by a kernel whose wait gave up
     uint64_t cap = 0;  // rows of the activation workspace
     bf16 *H1 = nullptr, *H2 = nullptr, *dZ2 = nullptr, *dZ1 = nullptr;
-    float *y = nullptr, *dy = nullptr, *loss = nullptr;
+    float *y = nullptr;     // partial sums of the outputs, HID / 32 per row
+    float *loss = nullptr;  // after the gradients, in their allocation
     uint64_t steps = 0;
     int loss_kind = ASSE_LOSS_LOG_MSE;
     // workspace of asse_report_learned, for rl_cap candidates
@@ -409,73 +452,56 @@ int ensure_workspace(asse_mlp *m, uint64_t rows)
     cudaFree(m->dZ2);
     cudaFree(m->dZ1);
     cudaFree(m->y);
-    cudaFree(m->dy);
     m->H1 = m->H2 = m->dZ2 = m->dZ1 = nullptr;
-    m->y = m->dy = nullptr;
+    m->y = nullptr;
     m->cap = 0;
     const size_t act = rows * HID * sizeof(bf16);
     MCK(m, cudaMalloc(&m->H1, act));
     MCK(m, cudaMalloc(&m->H2, act));
     MCK(m, cudaMalloc(&m->dZ2, act));
     MCK(m, cudaMalloc(&m->dZ1, act));
-    MCK(m, cudaMalloc(&m->y, rows * sizeof(float)));
-    MCK(m, cudaMalloc(&m->dy, rows * sizeof(float)));
+    MCK(m, cudaMalloc(&m->y, rows * (HID / 32) * sizeof(float)));
     m->cap = rows;
     return ASSE_OK;
 }
 
-// Forward pass of n rows into y (and H1, H2 kept for the backward pass).
-int forward(asse_mlp *m, const bf16 *x, uint64_t n, float *y, bool keep)
-{
-    const float *P = m->params;
-    MCK(m, cudaGetLastError());
-    fill_kernel<<<(unsigned)((n + 255) / 256 < 1024 ? (n + 255) / 256 : 1024), 256, 0, m->stream>>>(y, n, P + OFF_B3);
-    m->launches++;
-    MCK(m, launch_tc_gemm(TcOperand{x, FEAT, 1}, TcOperand{m->w1b, FEAT, 1}, (int)n, HID, FEAT, 1,
-                          TcEpi{TE_BIAS_RELU, P + OFF_B1, nullptr, nullptr, m->H1, nullptr, nullptr, HID}, m->error,
-                          m->stream, &m->launches));
-    MCK(m, launch_tc_gemm(TcOperand{m->H1, HID, 1}, TcOperand{m->w2b, HID, 1}, (int)n, HID, HID, 1,
-                          TcEpi{TE_BIAS_RELU_DOT, P + OFF_B2, P + OFF_W3, nullptr, keep ? m->H2 : nullptr, nullptr, y,
-                                HID},
-                          m->error, m->stream, &m->launches));
-    return ASSE_OK;
-}
-
+// The gradients of the mean loss of n rows: five launches.
 int backward(asse_mlp *m, const bf16 *x, const float *t, uint64_t n, float *loss_dev)
 {
     if (int rc = ensure_workspace(m, n))
         return rc;
-    if (int rc = forward(m, x, n, m->y, true))
-        return rc;
+    const float *P = m->params;
     float *G = m->grads;
-    MCK(m, cudaMemsetAsync(G, 0, NPARAMS * sizeof(float), m->stream));
-    MCK(m, cudaMemsetAsync(m->loss, 0, sizeof(float), m->stream));
-    const unsigned eb = (unsigned)((n + 255) / 256 < 1024 ? (n + 255) / 256 : 1024);
-    loss_kernel<<<eb, 256, 0, m->stream>>>(m->y, t, n, m->loss_kind, m->dy, m->loss);
-    const unsigned rb = (unsigned)(n < 2048 ? n : 2048);
-    out_grad_kernel<<<rb, HID, 0, m->stream>>>(m->dy, m->H2, m->params + OFF_W3, n, m->dZ2, G + OFF_W3, G + OFF_B2,
-                                              G + OFF_B3);
-    m->launches += 2;
+    MCK(m, cudaGetLastError());
+    const TcExtra nothing{};
+    // the first launch also zeroes the gradients and the loss
+    const TcProduct h1{TcOperand{x, FEAT, 1}, TcOperand{m->w1b, FEAT, 1}, (int)n, HID, FEAT, 1,
+                       TcEpi{TE_BIAS_RELU, P + OFF_B1, nullptr, nullptr, m->H1, nullptr, nullptr, HID}};
+    MCK(m, launch_tc_gemm(&h1, 1, TcExtra{G, (uint32_t)NPARAMS + 1, nullptr, nullptr}, m->error, m->stream,
+                          &m->launches));
+    const TcProduct h2{TcOperand{m->H1, HID, 1}, TcOperand{m->w2b, HID, 1}, (int)n, HID, HID, 1,
+                       TcEpi{TE_BIAS_RELU_DOT, P + OFF_B2, P + OFF_W3, nullptr, m->H2, nullptr, m->y, HID}};
+    MCK(m, launch_tc_gemm(&h2, 1, nothing, m->error, m->stream, &m->launches));
+    const uint64_t ob = (n + OUT_ROWS - 1) / OUT_ROWS;
+    out_grad_kernel<<<(unsigned)(ob < 608 ? ob : 608), 256, 0, m->stream>>>(
+        m->y, P + OFF_B3, t, n, m->loss_kind, m->H2, P + OFF_W3, m->dZ2, G + OFF_W3, G + OFF_B2, G + OFF_B3, m->loss);
+    m->launches++;
     MCK(m, cudaGetLastError());
     // the weight-gradient products reduce over the batch: split it so that
     // enough CTAs share the work
     const int splits = (int)((n + 255) / 256);
-    // dW2[o][i] = sum_m dZ2[m][o] H1[m][i]
-    MCK(m, launch_tc_gemm(TcOperand{m->dZ2, 1, HID}, TcOperand{m->H1, 1, HID}, HID, HID, (int)n, splits,
-                          TcEpi{TE_ATOMIC, nullptr, nullptr, nullptr, nullptr, G + OFF_W2, nullptr, HID}, m->error,
-                          m->stream, &m->launches));
-    // dZ1 = (dZ2 W2) masked by H1 > 0
-    MCK(m, launch_tc_gemm(TcOperand{m->dZ2, HID, 1}, TcOperand{m->w2b, 1, HID}, (int)n, HID, HID, 1,
-                          TcEpi{TE_RELU_GRAD, nullptr, nullptr, m->H1, m->dZ1, nullptr, nullptr, HID}, m->error,
-                          m->stream, &m->launches));
-    colsum_kernel<<<rb, HID, 0, m->stream>>>(m->dZ1, n, G + OFF_B1);
-    m->launches++;
-    // dW1[o][j] = sum_m dZ1[m][o] X[m][j]
-    MCK(m, launch_tc_gemm(TcOperand{m->dZ1, 1, HID}, TcOperand{x, 1, FEAT}, HID, FEAT, (int)n, splits,
-                          TcEpi{TE_ATOMIC, nullptr, nullptr, nullptr, nullptr, G + OFF_W1, nullptr, FEAT}, m->error,
-                          m->stream, &m->launches));
-    if (loss_dev)
-        MCK(m, cudaMemcpyAsync(loss_dev, m->loss, sizeof(float), cudaMemcpyDeviceToDevice, m->stream));
+    const TcProduct hidden[2] = {
+        // dW2[o][i] = sum_m dZ2[m][o] H1[m][i]
+        {TcOperand{m->dZ2, 1, HID}, TcOperand{m->H1, 1, HID}, HID, HID, (int)n, splits,
+         TcEpi{TE_ATOMIC, nullptr, nullptr, nullptr, nullptr, G + OFF_W2, nullptr, HID}},
+        // dZ1 = (dZ2 W2) masked by H1 > 0, db1 its column sums
+        {TcOperand{m->dZ2, HID, 1}, TcOperand{m->w2b, 1, HID}, (int)n, HID, HID, 1,
+         TcEpi{TE_RELU_GRAD, nullptr, nullptr, m->H1, m->dZ1, G + OFF_B1, nullptr, HID}}};
+    MCK(m, launch_tc_gemm(hidden, 2, nothing, m->error, m->stream, &m->launches));
+    // dW1[o][j] = sum_m dZ1[m][o] X[m][j]; this launch also hands the loss out
+    const TcProduct w1{TcOperand{m->dZ1, 1, HID}, TcOperand{x, 1, FEAT}, HID, FEAT, (int)n, splits,
+                       TcEpi{TE_ATOMIC, nullptr, nullptr, nullptr, nullptr, G + OFF_W1, nullptr, FEAT}};
+    MCK(m, launch_tc_gemm(&w1, 1, TcExtra{nullptr, 0, loss_dev, m->loss}, m->error, m->stream, &m->launches));
     return ASSE_OK;
 }
 
@@ -695,12 +721,12 @@ int asse_mlp_create(uint64_t seed, void *stream, asse_mlp **out)
             e = cudaMalloc(p, b);
     };
     alloc((void **)&m->params, NPARAMS * sizeof(float));
-    alloc((void **)&m->grads, NPARAMS * sizeof(float));
+    alloc((void **)&m->grads, (NPARAMS + 1) * sizeof(float));
+    m->loss = m->grads + NPARAMS;
     alloc((void **)&m->m1, NPARAMS * sizeof(float));
     alloc((void **)&m->m2, NPARAMS * sizeof(float));
     alloc((void **)&m->w1b, (size_t)HID * FEAT * sizeof(bf16));
     alloc((void **)&m->w2b, (size_t)HID * HID * sizeof(bf16));
-    alloc((void **)&m->loss, sizeof(float));
     alloc((void **)&m->w1p, (size_t)HID * FEAT * sizeof(bf16));
     alloc((void **)&m->w2p, (size_t)HID * HID * sizeof(bf16));
     alloc((void **)&m->error, sizeof(int));
@@ -750,8 +776,8 @@ void asse_mlp_destroy(asse_mlp *m)
         return;
     cudaStreamSynchronize(m->stream);
     for (void *p : {(void *)m->params, (void *)m->grads, (void *)m->m1, (void *)m->m2, (void *)m->w1b, (void *)m->w2b,
-                    (void *)m->H1, (void *)m->H2, (void *)m->dZ2, (void *)m->dZ1, (void *)m->y, (void *)m->dy,
-                    (void *)m->loss, (void *)m->w1p, (void *)m->w2p, (void *)m->error, (void *)m->rl})
+                    (void *)m->H1, (void *)m->H2, (void *)m->dZ2, (void *)m->dZ1, (void *)m->y,
+                    (void *)m->w1p, (void *)m->w2p, (void *)m->error, (void *)m->rl})
         cudaFree(p);
     delete m;
 }
@@ -829,11 +855,10 @@ int asse_mlp_train_step(asse_mlp *m, const uint16_t *x_dev, const float *t_dev, 
         return rc;
     m->steps++;
     const float b1t = 1.0f - powf(0.9f, (float)m->steps), b2t = 1.0f - powf(0.999f, (float)m->steps);
-    adam_kernel<<<128, 256, 0, m->stream>>>(m->params, m->grads, m->m1, m->m2, NPARAMS, lr, b1t, b2t, m->w1b,
-                                           m->w2b);
+    adam_kernel<<<(unsigned)((NPARAMS + 255) / 256), 256, 0, m->stream>>>(
+        m->params, m->grads, m->m1, m->m2, NPARAMS, lr, b1t, b2t, m->w1b, m->w2b, m->w1p, m->w2p);
     m->launches++;
     MCK(m, cudaGetLastError());
-    MCK(m, launch_mlp_pack(m->params, m->w1p, m->w2p, m->stream, &m->launches));
     return ASSE_OK;
 }
 

@@ -185,13 +185,10 @@ __global__ void pack_kernel(const float *params, bf16 *w1p, bf16 *w2p)
     const uint32_t n1 = HID * FEAT, n2 = HID * HID;
     for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n1 + n2; i += gridDim.x * blockDim.x) {
         if (i < n1) {
-            const uint32_t n = i / FEAT, k = i % FEAT;
-            const uint32_t j = k / 16, kg = (k % 16) / 8;
-            w1p[j * (HID * 16) + (n / 8) * 128 + kg * 64 + (n % 8) * 8 + (k % 8)] = __float2bfloat16_rn(params[i]);
+            w1p[mlp_w1p_at(i / FEAT, i % FEAT)] = __float2bfloat16_rn(params[i]);
         } else {
-            const uint32_t e = i - n1, n = e / HID, k = e % HID;
-            w2p[(n / 8) * (HID * 8) + (k / 8) * 64 + (n % 8) * 8 + (k % 8)] =
-                __float2bfloat16_rn(params[P_B1 + HID + e]);
+            const uint32_t e = i - n1;
+            w2p[mlp_w2p_at(e / HID, e % HID)] = __float2bfloat16_rn(params[P_B1 + HID + e]);
         }
     }
 }
@@ -403,23 +400,50 @@ __global__ void __launch_bounds__(THREADS, 1)
 // ---------------------------------------------------------------- training GEMMs
 
 // C[M][N] = sum_k A(m, k) B(n, k) for the products of the training pass, on
-// the tensor cores.  One CTA of four warps computes a 128 x BN tile (BN = 64,
-// or N when N is not a multiple of 64; N <= 256, a multiple of 16) over the
-// k range of blockIdx.z; A and B are gathered
-// from global memory through their (row, k) strides into the K-major
-// core-matrix layout in shared memory (the weight-gradient products read
-// their operands transposed), 64 k at a time through two stages; one thread
-// issues the MMAs (M = 128, N, K = 16) into a tensor-memory accumulator and
-// commits each stage to an mbarrier, so the gather of the next stage overlaps
-// the MMAs of this one.  The epilogue reads the accumulator with tcgen05.ld
-// (warp w: rows 32 w ..) and applies the step's fused operation.
-constexpr int TG_THREADS = 128;
+// the tensor cores.  One CTA of eight warps computes a 128 x BN tile (BN = 64,
+// or N when N is not a multiple of 64; N <= 256, a multiple of 16) over a k
+// range, 64 k at a time through four stages; one thread issues the MMAs
+// (M = 128, N, K = 16) into a tensor-memory accumulator and commits each stage
+// to an mbarrier.  The products of a training batch are small (a k range of 80
+// to 256), so what bounds a launch is latency, and the operands are read with
+// as much in flight as there is:
+//  * rows contiguous in k go to shared memory with 16-byte cp.async, up to four
+//    chunks ahead;
+//  * rows contiguous in the row index (the weight gradients read both operands
+//    transposed) are read 8 x 8 elements a thread, eight 16-byte loads one
+//    chunk ahead, and transposed in registers (32 byte permutations);
+//  * any other strides are gathered element by element.
+// In shared memory a core matrix (8 rows x 16 bytes) of k-group kg and row group
+// rb lies at 1152 rb + 144 kg: with 144 bytes between k-groups instead of 128
+// the stores of both kinds fall in distinct bank groups.
+// The epilogue reads the accumulator with tcgen05.ld (warp w: rows 32 (w mod 4),
+// every other 32 columns) and applies the step's fused operation with 16-byte
+// accesses.  Two independent products share a launch (TcJobs).
+// Four Adam steps of 4,096 rows and the parameters read back: 1,073 -> 266 us
+// (with the epilogues and the launches around, asse_learn.cu: 16 -> 6 a step);
+// the products took 35 us each with 2-byte gathers and stores.
+constexpr int TG_THREADS = 256;
 constexpr int TG_KC = 64;                               // k per stage
-constexpr uint32_t TG_A = 128 * TG_KC * 2;              // 16 KB
-constexpr uint32_t TG_B = 256 * TG_KC * 2;              // 32 KB
-constexpr uint32_t TG_BAR = 2 * (TG_A + TG_B);          // 2 stage barriers + final barrier + tmem slot, abort
-constexpr uint32_t TG_SMEM = TG_BAR + 64 + 1024;        // + alignment slack of the base
-constexpr uint32_t TG_TMEM_COLS = 256;
+constexpr int TG_STAGES = 4;
+constexpr uint32_t TG_LBO = 144, TG_SBO = 8 * TG_LBO;   // between k-groups, between groups of 8 rows
+constexpr uint32_t TG_A = 128 / 8 * TG_SBO;             // 18 KB
+
+enum { TG_ANY = 0, TG_ROWS = 1, TG_COLS = 2 };          // how an operand is read (above)
+
+// Bytes of a stage, of a CTA whose B tile has bn rows.
+__host__ __device__ constexpr uint32_t tg_stage(int bn) { return TG_A + (uint32_t)bn / 8 * TG_SBO; }
+
+struct TcPlan {
+    TcProduct p;
+    int BN, kchunk, nx, ny, amode, bmode;
+};
+struct TcPlans {
+    TcPlan j[2];
+    int first;         // CTAs of j[0]
+    uint32_t bar;      // byte offset of the barriers
+    uint32_t columns;  // tensor-memory columns of a CTA
+    TcExtra extra;
+};
 
 __device__ __forceinline__ void mma_f16_n(uint32_t d_tmem, uint64_t a, uint64_t b, uint32_t idesc,
                                           uint32_t accumulate)
@@ -447,65 +471,160 @@ __device__ __forceinline__ void tmem_ld32(uint32_t taddr, float *v)
         v[i] = __uint_as_float(r[i]);
 }
 
-// Gather rows [r0, r0 + rows) x k [k0, k0 + 64) of an operand into the
-// K-major core-matrix layout: element (row, k) at byte
-// (row / 8) * 1024 + (k / 8) * 128 + (row % 8) * 16 + (k % 8) * 2; outside
-// [0, nrows) x [k0, kend) zero.  Rows contiguous in k (sk = 1, 16-byte
-// aligned groups) move as one 16-byte load per 8 k; otherwise each thread
-// takes consecutive rows so that the warp's loads of one k are contiguous
-// when the operand is row-contiguous (si = 1).
-__device__ __forceinline__ void tg_gather(uint8_t *dst, TcOperand op, int r0, int rows, int nrows, int k0, int kend)
+__device__ __forceinline__ void cp_async16(uint32_t dst, const void *src, bool ok)
 {
-    const bool vec = op.sk == 1 && (op.si % 8) == 0 && (reinterpret_cast<uintptr_t>(op.p) & 15u) == 0;
+    // with a source size of 0 the 16 bytes are zeros
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(ok ? 16 : 0) : "memory");
+}
+
+// Where element group (row, k-group kg) of a tile lies.
+__device__ __forceinline__ uint32_t tg_at(int row, int kg)
+{
+    return (uint32_t)(row >> 3) * TG_SBO + (uint32_t)kg * TG_LBO + (uint32_t)(row & 7) * 16;
+}
+
+// Rows [r0, r0 + rows) x k [k0, k0 + 64) of an operand contiguous in k (K and
+// kend multiples of 8); zeros outside [0, nrows) x [k0, kend).
+__device__ __forceinline__ void tg_rows(uint32_t dst, const TcOperand &op, int r0, int rows, int nrows, int k0, int kend)
+{
     for (int e = threadIdx.x; e < rows * (TG_KC / 8); e += TG_THREADS) {
-        const int row = vec ? e / (TG_KC / 8) : e % rows;
-        const int kg = vec ? e % (TG_KC / 8) : e / rows;
+        const int row = e / (TG_KC / 8), kg = e % (TG_KC / 8);
         const int i = r0 + row, k = k0 + kg * 8;
-        uint4 v = make_uint4(0, 0, 0, 0);
-        if (i < nrows) {
-            if (vec && k + 8 <= kend) {
-                v = *reinterpret_cast<const uint4 *>(op.p + (long)i * op.si + k);
-            } else {
-                uint16_t h[8];
-#pragma unroll
-                for (int j = 0; j < 8; j++)
-                    h[j] = k + j < kend ? __bfloat16_as_ushort(op.p[(long)i * op.si + (long)(k + j) * op.sk]) : 0;
-                v = make_uint4(h[0] | ((uint32_t)h[1] << 16), h[2] | ((uint32_t)h[3] << 16),
-                               h[4] | ((uint32_t)h[5] << 16), h[6] | ((uint32_t)h[7] << 16));
-            }
-        }
-        *reinterpret_cast<uint4 *>(dst + (row >> 3) * 1024 + kg * 128 + (row & 7) * 16) = v;
+        const bool ok = i < nrows && k < kend;
+        cp_async16(dst + tg_at(row, kg), ok ? op.p + (long)i * op.si + k : op.p, ok);
     }
 }
 
-// The CTA at (x, y, z) computes rows 128 x .. and columns BN y .. BN y + BN - 1
-// over the z-th k range.
-__global__ void __launch_bounds__(TG_THREADS) tc_gemm_kernel(TcOperand A, TcOperand B, int M, int N, int BN, int K,
-                                                             int kchunk, TcEpi epi, int *error)
+// The same of an operand of any strides, element by element.
+__device__ __forceinline__ void tg_any(uint8_t *dst, const TcOperand &op, int r0, int rows, int nrows, int k0, int kend)
+{
+    for (int e = threadIdx.x; e < rows * (TG_KC / 8); e += TG_THREADS) {
+        const int row = e % rows, kg = e / rows;
+        const int i = r0 + row, k = k0 + kg * 8;
+        uint16_t h[8];
+#pragma unroll
+        for (int j = 0; j < 8; j++)
+            h[j] = i < nrows && k + j < kend ? __bfloat16_as_ushort(op.p[(long)i * op.si + (long)(k + j) * op.sk]) : 0;
+        *reinterpret_cast<uint4 *>(dst + tg_at(row, kg)) =
+            make_uint4(h[0] | ((uint32_t)h[1] << 16), h[2] | ((uint32_t)h[3] << 16), h[4] | ((uint32_t)h[5] << 16),
+                       h[6] | ((uint32_t)h[7] << 16));
+    }
+}
+
+// A thread's 8 x 8 block of an operand contiguous in the row index: row v[kk]
+// of the block in memory holds k-group element kk of its eight rows.
+__device__ __forceinline__ void tg_cols_load(uint4 (&v)[8], const bf16 *p, long sk, int k, int kend)
+{
+#pragma unroll
+    for (int kk = 0; kk < 8; kk++)
+        v[kk] = p != nullptr && k + kk < kend ? *reinterpret_cast<const uint4 *>(p + (long)(k + kk) * sk)
+                                              : make_uint4(0, 0, 0, 0);
+}
+
+__device__ __forceinline__ void tg_cols_store(uint8_t *dst, const uint4 (&v)[8])
+{
+#pragma unroll
+    for (int r = 0; r < 8; r++) {
+        uint32_t w[4];
+#pragma unroll
+        for (int m = 0; m < 4; m++)
+            w[m] = __byte_perm(u4get(v[2 * m], r / 2), u4get(v[2 * m + 1], r / 2), r & 1 ? 0x7632 : 0x5410);
+        *reinterpret_cast<uint4 *>(dst + r * 16) = make_uint4(w[0], w[1], w[2], w[3]);
+    }
+}
+
+// Column sums over the warp's 32 rows of a 32 x 32 tile (v: this lane's row):
+// lane l returns the sum of column l.
+__device__ __forceinline__ float warp_column_sums(float (&v)[32], int lane)
+{
+#pragma unroll
+    for (int w = 16; w >= 1; w >>= 1) {
+        const bool up = (lane & w) != 0;
+#pragma unroll
+        for (int j = 0; j < w; j++) {
+            const float give = up ? v[j] : v[j + w], keep = up ? v[j + w] : v[j];
+            v[j] = keep + __shfl_xor_sync(FULL_MASK, give, w);
+        }
+    }
+    return v[0];
+}
+
+__global__ void __launch_bounds__(TG_THREADS, 2) tc_gemm_kernel(const __grid_constant__ TcPlans plans, int *error)
 {
     extern __shared__ uint8_t tg_raw[];
     uint8_t *sm = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(tg_raw) + 1023) & ~uintptr_t(1023));
-    uint64_t *bar = reinterpret_cast<uint64_t *>(sm + TG_BAR);  // [0], [1] stages, [2] final
-    volatile uint32_t *tmem_slot = reinterpret_cast<volatile uint32_t *>(bar + 3);
+    uint64_t *bar = reinterpret_cast<uint64_t *>(sm + plans.bar);  // stages, then the final one
+    volatile uint32_t *tmem_slot = reinterpret_cast<volatile uint32_t *>(bar + TG_STAGES + 1);
     volatile uint32_t *abort_flag = tmem_slot + 1;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int m0 = blockIdx.x * 128, n0 = blockIdx.y * BN;
-    const int kb = blockIdx.z * kchunk, ke = min(K, kb + kchunk);
+    const bool second = (int)blockIdx.x >= plans.first;
+    const TcPlan &J = plans.j[second ? 1 : 0];
+    const TcEpi &epi = J.p.epi;
+    const int M = J.p.M, N = J.p.N, BN = J.BN;
+    const int blk = (int)blockIdx.x - (second ? plans.first : 0);
+    const int m0 = blk % J.nx * 128, ny = blk / J.nx % J.ny, n0 = ny * BN, z = blk / (J.nx * J.ny);
+    const int kb = z * J.kchunk, ke = min(J.p.K, kb + J.kchunk);
     const int nchunks = ke > kb ? (ke - kb + TG_KC - 1) / TG_KC : 0;
+    if (plans.extra.zero)
+        for (uint32_t i = blockIdx.x * TG_THREADS + tid; i < plans.extra.n_zero; i += gridDim.x * TG_THREADS)
+            plans.extra.zero[i] = 0.0f;
+    if (plans.extra.to && blockIdx.x == 0 && tid == 0)
+        *plans.extra.to = *plans.extra.from;
     if (tid == 0) {
-        mbar_init(&bar[0], 1);
-        mbar_init(&bar[1], 1);
-        mbar_init(&bar[2], 1);
+        for (int i = 0; i <= TG_STAGES; i++)
+            mbar_init(&bar[i], 1);
         tmem_slot[1] = 0u;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     if (warp == 0) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
                          smem_addr(const_cast<uint32_t *>(tmem_slot))),
-                     "r"(TG_TMEM_COLS)
+                     "r"(plans.columns)
                      : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
+    // this thread's 8 x 8 block of a transposed operand: of A in threads
+    // 0..127, of B in the next BN (the first BN if A is not transposed)
+    const bf16 *tp = nullptr;
+    long tsk = 0;
+    int tkg = 0;
+    uint32_t tdst = 0;
+    bool tblock = false;
+    {
+        const int skip = J.amode == TG_COLS ? 128 : 0;
+        if (J.amode == TG_COLS && tid < 128) {
+            tblock = true;
+            tkg = tid & 7;
+            tsk = J.p.A.sk;
+            tdst = tg_at(tid / 8 * 8, tkg);
+            tp = m0 + tid / 8 * 8 < M ? J.p.A.p + m0 + tid / 8 * 8 : nullptr;
+        } else if (J.bmode == TG_COLS && tid >= skip && tid < skip + BN) {
+            const int t = tid - skip;
+            tblock = true;
+            tkg = t & 7;
+            tsk = J.p.B.sk;
+            tdst = TG_A + tg_at(t / 8 * 8, tkg);
+            tp = n0 + t / 8 * 8 < N ? J.p.B.p + n0 + t / 8 * 8 : nullptr;
+        }
+    }
+    const uint32_t stage_bytes = tg_stage(BN);
+    auto issue = [&](int c) {
+        const uint32_t st = smem_addr(sm + (c % TG_STAGES) * stage_bytes);
+        const int k0 = kb + c * TG_KC;
+        if (J.amode == TG_ROWS)
+            tg_rows(st, J.p.A, m0, 128, M, k0, ke);
+        if (J.bmode == TG_ROWS)
+            tg_rows(st + TG_A, J.p.B, n0, BN, N, k0, ke);
+    };
+    uint4 tv[8];
+#pragma unroll
+    for (int c = 0; c < TG_STAGES - 1; c++) {
+        if (c < nchunks)
+            issue(c);
+        asm volatile("cp.async.commit_group;" ::: "memory");
+    }
+    if (tblock)
+        tg_cols_load(tv, tp, tsk, kb + tkg * 8, ke);
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
@@ -513,74 +632,118 @@ __global__ void __launch_bounds__(TG_THREADS) tc_gemm_kernel(TcOperand A, TcOper
     // FP32 accumulator, BF16 A and B, both K-major, N >> 3, M = 128
     const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(BN >> 3) << 17) | ((128u >> 4) << 24);
     bool ok = true;
-    for (int c = 0; c < nchunks && ok; c++) {
-        const int s = c & 1;
-        // the stage is free once the MMAs of the chunk two back have read it
-        if (c >= 2 && !__syncthreads_and(wait_or_abort(&bar[s], ((c - 2) >> 1) & 1, abort_flag))) {
-            ok = false;
-            break;
+    for (int c = 0; c < nchunks; c++) {
+        const int s = c % TG_STAGES, nx = c + TG_STAGES - 1;
+        if (nx < nchunks) {
+            // the stage is free once the MMAs of the chunk TG_STAGES back have read it
+            if (nx >= TG_STAGES &&
+                !__syncthreads_and(wait_or_abort(&bar[nx % TG_STAGES], ((nx - TG_STAGES) / TG_STAGES) & 1, abort_flag))) {
+                ok = false;
+                break;
+            }
+            issue(nx);
         }
-        uint8_t *sa = sm + s * (TG_A + TG_B), *sb = sa + TG_A;
+        asm volatile("cp.async.commit_group;" ::: "memory");
+        uint8_t *sa = sm + s * stage_bytes, *sb = sa + TG_A;
         const int k0 = kb + c * TG_KC;
-        tg_gather(sa, A, m0, 128, M, k0, ke);
-        tg_gather(sb, B, n0, BN, N, k0, ke);
+        if (tblock) {
+            tg_cols_store(sa + tdst, tv);
+            if (c + 1 < nchunks)
+                tg_cols_load(tv, tp, tsk, k0 + TG_KC + tkg * 8, ke);
+        }
+        if (J.amode == TG_ANY)
+            tg_any(sa, J.p.A, m0, 128, M, k0, ke);
+        if (J.bmode == TG_ANY)
+            tg_any(sb, J.p.B, n0, BN, N, k0, ke);
+        asm volatile("cp.async.wait_group %0;" ::"n"(TG_STAGES - 1) : "memory");
         fence_async_smem();  // the generic stores before the tensor core reads them
         tc_fence_before();
         __syncthreads();
         if (tid == 0) {
             tc_fence_after();
             const uint32_t ab = smem_addr(sa), bb = smem_addr(sb);
-#pragma unroll
-            for (int kk = 0; kk < TG_KC / 16; kk++)
-                mma_f16_n(tmem, sdesc(ab + kk * 256, 128, 1024), sdesc(bb + kk * 256, 128, 1024), idesc,
-                          (c > 0 || kk > 0) ? 1u : 0u);
+            const int steps = min(TG_KC / 16, (ke - k0 + 15) / 16);
+            for (int kk = 0; kk < steps; kk++)
+                mma_f16_n(tmem, sdesc(ab + kk * 2 * TG_LBO, TG_LBO, TG_SBO), sdesc(bb + kk * 2 * TG_LBO, TG_LBO, TG_SBO),
+                          idesc, (c > 0 || kk > 0) ? 1u : 0u);
             mma_commit(&bar[s]);
         }
     }
+    asm volatile("cp.async.wait_all;" ::: "memory");
     // every MMA done (or none issued) before the accumulator is read or freed
-    if (tid == 0) {
-        mma_commit(&bar[2]);
-    }
-    const bool done = __syncthreads_and(ok && wait_or_abort(&bar[2], 0, abort_flag));
+    if (tid == 0)
+        mma_commit(&bar[TG_STAGES]);
+    const bool done = __syncthreads_and(ok && wait_or_abort(&bar[TG_STAGES], 0, abort_flag));
     if (!done && tid == 0)
-        mbar_wait(&bar[2], 0);  // bounded: the committed MMAs finish before the free below
+        mbar_wait(&bar[TG_STAGES], 0);  // bounded: the committed MMAs finish before the free below
     tc_fence_after();
     if (done && nchunks > 0) {
-        const int m = m0 + warp * 32 + lane;
-        float dot = 0.0f;
-        for (int cb = 0; cb < BN; cb += 32) {
+        const int m = m0 + (warp & 3) * 32 + lane;
+        const long row = (long)m * epi.ld;
+        for (int cb = warp / 4 * 32; cb < BN; cb += 64) {
             float v[32];
-            tmem_ld32(tmem + ((uint32_t)(warp * 32) << 16) + cb, v);
-            if (m >= M)
-                continue;
+            __syncwarp();
+            tmem_ld32(tmem + ((uint32_t)((warp & 3) * 32) << 16) + cb, v);
+            const int n = n0 + cb, cols = min(32, min(BN - cb, N - n));  // a multiple of 16
+            if (epi.kind == TE_ATOMIC) {
+                if (m < M)
 #pragma unroll
-            for (int j = 0; j < 32; j++) {
-                const int n = n0 + cb + j;
-                if (cb + j >= BN || n >= N)
-                    break;
-                const float a = v[j];
-                if (epi.kind == TE_ATOMIC) {
-                    atomicAdd(&epi.outf[(long)m * epi.ld + n], a);
-                } else if (epi.kind == TE_RELU_GRAD) {
-                    const float act = __bfloat162float(epi.act[(long)m * epi.ld + n]);
-                    epi.out[(long)m * epi.ld + n] = __float2bfloat16_rn(act > 0.0f ? a : 0.0f);
+                    for (int j = 0; j < 32; j += 4)
+                        if (j < cols)
+                            atomicAdd(reinterpret_cast<float4 *>(epi.outf + row + n + j),
+                                      make_float4(v[j], v[j + 1], v[j + 2], v[j + 3]));
+                continue;
+            }
+            float dot = 0.0f;
+#pragma unroll
+            for (int j = 0; j < 32; j += 8) {
+                if (j >= cols || m >= M) {
+#pragma unroll
+                    for (int i = 0; i < 8; i++)
+                        v[j + i] = 0.0f;
+                    continue;
+                }
+                uint32_t w[4];
+                if (epi.kind == TE_RELU_GRAD) {
+                    const uint4 act = *reinterpret_cast<const uint4 *>(epi.act + row + n + j);
+#pragma unroll
+                    for (int i = 0; i < 4; i++) {
+                        const __nv_bfloat162 h = *reinterpret_cast<const __nv_bfloat162 *>(
+                            i == 0 ? &act.x : i == 1 ? &act.y : i == 2 ? &act.z : &act.w);
+                        w[i] = pack_bf16x2(__low2float(h) > 0.0f ? v[j + 2 * i] : 0.0f,
+                                           __high2float(h) > 0.0f ? v[j + 2 * i + 1] : 0.0f);
+                    }
                 } else {
-                    const bf16 h = __float2bfloat16_rn(fmaxf(a + epi.bias[n], 0.0f));
-                    if (epi.out)
-                        epi.out[(long)m * epi.ld + n] = h;
+#pragma unroll
+                    for (int i = 0; i < 4; i++)
+                        w[i] = pack_bf16x2(fmaxf(v[j + 2 * i] + epi.bias[n + j + 2 * i], 0.0f),
+                                           fmaxf(v[j + 2 * i + 1] + epi.bias[n + j + 2 * i + 1], 0.0f));
+                }
+                *reinterpret_cast<uint4 *>(epi.out + row + n + j) = make_uint4(w[0], w[1], w[2], w[3]);
+                // the stored values, for the dot product or the column sums
+#pragma unroll
+                for (int i = 0; i < 4; i++) {
+                    v[j + 2 * i] = __uint_as_float(w[i] << 16);
+                    v[j + 2 * i + 1] = __uint_as_float(w[i] & 0xffff0000u);
                     if (epi.kind == TE_BIAS_RELU_DOT)
-                        dot = fmaf(__bfloat162float(h), epi.w3[n], dot);
+                        dot = fmaf(v[j + 2 * i + 1], epi.w3[n + j + 2 * i + 1],
+                                   fmaf(v[j + 2 * i], epi.w3[n + j + 2 * i], dot));
                 }
             }
+            if (epi.kind == TE_BIAS_RELU_DOT && m < M)
+                epi.y[(long)(n / 32) * M + m] = dot;
+            if (epi.kind == TE_RELU_GRAD) {
+                const float s = warp_column_sums(v, lane);
+                if (lane < cols)
+                    atomicAdd(&epi.outf[n + lane], s);
+            }
         }
-        if (epi.kind == TE_BIAS_RELU_DOT && m < M)
-            atomicAdd(&epi.y[m], dot);
     }
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
     if (warp == 0)
-        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(TG_TMEM_COLS)
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(plans.columns)
                      : "memory");
     if (tid == 0 && (!done || tmem_slot[1] != 0u))
         atomicExch(error, 1);
@@ -608,19 +771,54 @@ EncodeTiled encode_fn()
 
 }  // namespace
 
-cudaError_t launch_tc_gemm(TcOperand A, TcOperand B, int M, int N, int K, int splits, const TcEpi &epi, int *error,
-                           cudaStream_t s, uint64_t *launches)
+static int tc_mode(const TcOperand &o, int rows, int K, int tile_rows)
 {
-    if (N < 16 || N > 256 || N % 16 != 0 || M < 1 || K < 1 || splits < 1)
+    if ((reinterpret_cast<uintptr_t>(o.p) & 15u) != 0)
+        return TG_ANY;
+    if (o.sk == 1 && o.si % 8 == 0 && K % 8 == 0)
+        return TG_ROWS;
+    if (o.si == 1 && o.sk % 8 == 0 && rows % 8 == 0 && tile_rows <= 128)
+        return TG_COLS;
+    return TG_ANY;
+}
+
+cudaError_t launch_tc_gemm(const TcProduct *products, int count, const TcExtra &extra, int *error, cudaStream_t s,
+                           uint64_t *launches)
+{
+    if (count < 1 || count > 2)
         return cudaErrorInvalidValue;
-    cudaError_t e = cudaFuncSetAttribute(tc_gemm_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TG_SMEM);
+    TcPlans plans{};
+    plans.extra = extra;
+    uint32_t stage = 0, grid = 0;
+    int bn = 0;
+    for (int i = 0; i < count; i++) {
+        TcPlan &J = plans.j[i];
+        const TcProduct &p = products[i];
+        if (p.N < 16 || p.N > 256 || p.N % 16 != 0 || p.M < 1 || p.K < 1 || p.splits < 1)
+            return cudaErrorInvalidValue;
+        J.p = p;
+        // 64-column tiles where N allows, for more CTAs on the small products of a training batch
+        J.BN = p.N % 64 == 0 ? 64 : p.N;
+        J.kchunk = ((p.K + p.splits - 1) / p.splits + TG_KC - 1) / TG_KC * TG_KC;
+        J.nx = (p.M + 127) / 128;
+        J.ny = (p.N + J.BN - 1) / J.BN;
+        J.amode = tc_mode(p.A, p.M, p.K, 128);
+        J.bmode = tc_mode(p.B, p.N, p.K, J.BN);
+        if (i == 0)
+            plans.first = J.nx * J.ny * ((p.K + J.kchunk - 1) / J.kchunk);
+        grid += (uint32_t)(J.nx * J.ny * ((p.K + J.kchunk - 1) / J.kchunk));
+        stage = stage > tg_stage(J.BN) ? stage : tg_stage(J.BN);
+        bn = bn > J.BN ? bn : J.BN;
+    }
+    plans.bar = TG_STAGES * stage;
+    plans.columns = 32;
+    while (plans.columns < (uint32_t)(bn + 31) / 32 * 32)  // whole 32-column loads
+        plans.columns *= 2;
+    const size_t smem = plans.bar + (TG_STAGES + 1) * 8 + 16 + 1024;  // + alignment slack of the base
+    cudaError_t e = cudaFuncSetAttribute(tc_gemm_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess)
         return e;
-    // 64-column tiles where N allows, for more CTAs on the small products of a training batch
-    const int BN = N % 64 == 0 ? 64 : N;
-    const int kchunk = ((K + splits - 1) / splits + TG_KC - 1) / TG_KC * TG_KC;
-    const dim3 grid((M + 127) / 128, (N + BN - 1) / BN, (K + kchunk - 1) / kchunk);
-    tc_gemm_kernel<<<grid, TG_THREADS, TG_SMEM, s>>>(A, B, M, N, BN, K, kchunk, epi, error);
+    tc_gemm_kernel<<<grid, TG_THREADS, smem, s>>>(plans, error);
     *launches += 1;
     return cudaGetLastError();
 }

@@ -7,6 +7,8 @@
 #include <cstdint>
 #include <string>
 
+#include "../../include/asse_learn.h"
+
 namespace asse {
 
 // fp32 parameters (asse_learn.h order) -> the packed BF16 operand images of
@@ -22,16 +24,28 @@ int launch_mlp_forward_tc(const __nv_bfloat16 *x, uint64_t n, const __nv_bfloat1
                           const float *params, float *y, int *error, cudaStream_t s, uint64_t *launches,
                           std::string *why);
 
+// Where element (n, k) of W1 [ASSE_HID][ASSE_FEAT] and of W2 [ASSE_HID][ASSE_HID]
+// lies in those images.
+__host__ __device__ inline uint32_t mlp_w1p_at(uint32_t n, uint32_t k)
+{
+    return k / 16 * (ASSE_HID * 16) + n / 8 * 128 + k % 16 / 8 * 64 + n % 8 * 8 + k % 8;
+}
+__host__ __device__ inline uint32_t mlp_w2p_at(uint32_t n, uint32_t k)
+{
+    return n / 8 * (ASSE_HID * 8) + k / 8 * 64 + n % 8 * 8 + k % 8;
+}
+
 // Products of the training pass on the tensor cores (tcgen05):
 // C[M][N] = sum_k A(m, k) B(n, k), operands addressed by strides (element
 // (i, k) at p[i * si + k * sk]), N a multiple of 16 up to 256, the k range
-// split over `splits` CTAs along z (only with TE_ATOMIC), and a fused
+// split over `splits` CTAs (more than one only with TE_ATOMIC), and a fused
 // epilogue:
 //   TE_BIAS_RELU      out = bf16(relu(C + bias[n]))
-//   TE_BIAS_RELU_DOT  the same (out may be null), and y[m] += sum_n out * w3[n]
-//   TE_RELU_GRAD      out = bf16(C) where act > 0, else 0
+//   TE_BIAS_RELU_DOT  the same, and y[n / 32][m] = the 32 columns' sum of out * w3[n]
+//   TE_RELU_GRAD      out = bf16(C) where act > 0, else 0, and outf[n] += its column sums
 //   TE_ATOMIC         outf[m][n] += C (FP32 atomics)
-// with row stride ld.  A CTA whose bounded wait gave up sets *error to 1.
+// with row stride ld (a multiple of 8; out, act and outf 16-byte aligned).  A
+// CTA whose bounded wait gave up sets *error to 1.
 struct TcOperand {
     const __nv_bfloat16 *p;
     long si, sk;
@@ -47,7 +61,21 @@ struct TcEpi {
     float *y;
     int ld;
 };
-cudaError_t launch_tc_gemm(TcOperand A, TcOperand B, int M, int N, int K, int splits, const TcEpi &epi, int *error,
-                           cudaStream_t s, uint64_t *launches);
+struct TcProduct {
+    TcOperand A, B;
+    int M, N, K, splits;
+    TcEpi epi;
+};
+// What a launch does besides (any of it null): n_zero floats at zero set to 0,
+// *to = *from.
+struct TcExtra {
+    float *zero;
+    uint32_t n_zero;
+    float *to;
+    const float *from;
+};
+// One launch of one product, or of two that do not depend on one another.
+cudaError_t launch_tc_gemm(const TcProduct *products, int count, const TcExtra &extra, int *error, cudaStream_t s,
+                           uint64_t *launches);
 
 }  // namespace asse
