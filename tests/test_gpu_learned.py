@@ -283,3 +283,27 @@ def test_synth_states_from_their_draws(mods, k, g, n):
         assert ln[si] == np.float32(np.log(d["card"]))
         want = -g * np.log((g - min(float(cnt), g - 0.5)) / g)
         assert abs(lc[si] - want) <= 1e-6 * want + 1e-6
+
+
+@pytest.mark.parametrize("n,shift", [(1, 0), (7, 0), (128, 0), (257, 0), (1031, 0), (130, 1), (65, 3)])
+def test_gradients_at_the_edges_of_the_tiles(mods, n, shift):
+    """Row counts around the products' 128-row tiles, 64-row chunks and 8-row
+    blocks, and feature rows that start off a 16-byte boundary (gathered element
+    by element), compared as the gradients above are."""
+    asse, oracle, omlp, torch = mods
+    m = asse.MLP(seed=9)
+    p = m.params().astype(np.float64)
+    rng = np.random.default_rng(n)
+    X = _bf16(np.abs(rng.normal(size=(n, 80))) * 0.3)
+    t = rng.normal(loc=5.0, scale=2.0, size=n)
+    flat = torch.zeros(n * 80 + shift, dtype=torch.bfloat16, device="cuda")
+    xd = flat[shift:].view(n, 80)
+    xd.copy_(torch.from_numpy(X.astype(np.float32)))
+    loss = float(m.backward(xd, torch.from_numpy(t.astype(np.float32)).cuda()).cpu()[0])
+    m.check()
+    g = m.grads().astype(np.float64)
+    loss_ref, g_ref, _ = omlp.loss_and_grads(p, X, t)
+    _ys, gs = omlp.error_scales(p, X, t)
+    assert abs(loss - loss_ref) <= 1e-3 * loss_ref
+    worst = np.abs(g - g_ref) / (gs + 1e-30)
+    assert worst.max() <= 2 ** -6, (int(worst.argmax()), worst.max())
