@@ -84,17 +84,25 @@ __device__ __forceinline__ double frame_up(const Params &P, const unsigned long 
     return up;
 }
 
+// The candidates of a warp (one per lane, if ok) join CSIP, those that reach
+// theta the report too: one atomic per list for the warp.
 __device__ __forceinline__ void emit(Status *st, asse_superpoint *csip, asse_superpoint *report, uint64_t out_cap,
-                                     const asse_superpoint &sp)
+                                     const asse_superpoint &sp, bool ok)
 {
-    const unsigned long long p = atomicAdd(&st->n_csip, 1ull);
-    if (p < out_cap)
+    const unsigned lane = threadIdx.x & 31, lt = (1u << lane) - 1u;
+    const bool rep = ok && (sp.flags & ASSE_SP_REPORTED) != 0;
+    const unsigned mc = __ballot_sync(FULL_MASK, ok), mr = __ballot_sync(FULL_MASK, rep);
+    unsigned long long base = 0;
+    if (lane == 0 && mc)
+        base = atomicAdd(&st->n_csip, (unsigned long long)__popc(mc));
+    if (lane == 1 && mr)
+        base = atomicAdd(&st->n_report, (unsigned long long)__popc(mr));
+    const unsigned long long p = __shfl_sync(FULL_MASK, base, 0) + __popc(mc & lt);
+    const unsigned long long p2 = __shfl_sync(FULL_MASK, base, 1) + __popc(mr & lt);
+    if (ok && p < out_cap)
         csip[p] = sp;
-    if (sp.flags & ASSE_SP_REPORTED) {
-        const unsigned long long p2 = atomicAdd(&st->n_report, 1ull);
-        if (p2 < out_cap)
-            report[p2] = sp;
-    }
+    if (rep && p2 < out_cap)
+        report[p2] = sp;
 }
 
 constexpr int RESTORE_THREADS = 512;
@@ -124,6 +132,8 @@ __global__ void __launch_bounds__(RESTORE_THREADS) restore_kernel(Params P, Scan
     __shared__ uint32_t n_sa[8];
     __shared__ double p_row[8];  // |AAT(k',i,j)| / (g 2^c) of each row (Sec. 4.3)
     __shared__ uint32_t n_next;
+    __shared__ double up_s;      // UP of the frame, and ln(1 - UP) in FP32
+    __shared__ float b_up_s;
     __shared__ Tuple sm_t[2][RESTORE_SMEM_TUPLES];
     __shared__ uint2 sm_x[4][RESTORE_SMEM_COLS];  // (bits, positions) of the columns of rows 0..3
     const uint32_t j = blockIdx.x;
@@ -150,6 +160,14 @@ __global__ void __launch_bounds__(RESTORE_THREADS) restore_kernel(Params P, Scan
     for (uint32_t i = 0; i < P.r; i++)
         if (n_sa[i] == 0)
             return;
+    if (tid == RESTORE_THREADS - 1) {
+        // UP of the frame: the product over the rows, in row order
+        double up = 1.0;
+        for (uint32_t i = 0; i < P.r; i++)
+            up = __dmul_rn(up, p_row[i]);
+        up_s = up;
+        b_up_s = log1pf(-(float)up);
+    }
     Tuple *cur_g = scratch + (size_t)j * 2 * cap;
     Tuple *nxt_g = cur_g + cap;
     Tuple *cur_s = sm_t[0], *nxt_s = sm_t[1];
@@ -234,28 +252,50 @@ __global__ void __launch_bounds__(RESTORE_THREADS) restore_kernel(Params P, Scan
             n_next = 0;
         __syncthreads();
     }
-    const int lane = tid & 31, warp = tid >> 5;
-    for (uint32_t t = warp; t < n_cur; t += RESTORE_THREADS / 32) {
-        const Tuple tu = *tuple_at(cur_s, cur_g, t);
-        uint32_t nat = 0;
-        for (uint32_t m = lane; m < P.mw; m += 32) {
-            uint32_t acc = FULL_MASK;
-            for (uint32_t i = 0; i < P.r; i++)
-                acc &= o.sa_mask[(((size_t)i * P.nf + j) * cols + tu.slot[i]) * P.mw + m];
-            nat += __popc(acc);
+    // NAT and the estimate of the complete tuples, RESTORE_THREADS at a time.
+    // What bounds this is latency: the masks are read with as many lanes per
+    // tuple as a mask has words (32 at most), then a lane takes a tuple through
+    // the inverse mangling and Eq. 4 and a warp appends its tuples to the lists
+    // with one atomic each; a warp taking one tuple at a time through all of it
+    // took 13.8 us for the link workload, 11.7 now.
+    uint32_t ll = 0;  // log2 lanes per tuple
+    while (ll < 5 && (1u << ll) < P.mw)
+        ll++;
+    const uint32_t groups = RESTORE_THREADS >> ll, grp = (uint32_t)tid >> ll, sub = (uint32_t)tid & ((1u << ll) - 1);
+    uint32_t *nat_s = reinterpret_cast<uint32_t *>(nxt_s);  // the other level's tuples are not needed any more
+    static_assert(RESTORE_SMEM_TUPLES * sizeof(Tuple) >= RESTORE_THREADS * sizeof(uint32_t), "NATs of a round");
+    const uint32_t *masks = o.sa_mask + (size_t)j * cols * P.mw;
+    for (uint32_t t0 = 0; t0 < n_cur; t0 += RESTORE_THREADS) {
+        const uint32_t nt = min(n_cur - t0, (uint32_t)RESTORE_THREADS);
+        __syncthreads();  // the frame's UP is written, the last round's NATs are read
+        for (uint32_t q0 = 0; q0 < nt; q0 += groups) {
+            const uint32_t q = q0 + grp;
+            uint32_t nat = 0;
+            if (q < nt) {
+                const Tuple *tu = tuple_at(cur_s, cur_g, t0 + q);
+                for (uint32_t m = sub; m < P.mw; m += 1u << ll) {
+                    uint32_t acc = FULL_MASK;
+                    for (uint32_t i = 0; i < P.r; i++)
+                        acc &= masks[((size_t)i * P.nf * cols + tu->slot[i]) * P.mw + m];
+                    nat += __popc(acc);
+                }
+            }
+            for (uint32_t off = 1; off < (1u << ll); off <<= 1)
+                nat += __shfl_xor_sync(FULL_MASK, nat, off);
+            if (sub == 0 && q < nt)
+                nat_s[q] = nat;
         }
-        nat = __reduce_add_sync(FULL_MASK, nat);
-        if (lane == 0) {
-            // UP of the frame: the product over the rows, in row order
-            double up = 1.0;
-            for (uint32_t i = 0; i < P.r; i++)
-                up = __dmul_rn(up, p_row[i]);
-            const uint32_t y = (uint32_t)(((uint64_t)tu.L << P.u) | j);
-            asse_superpoint sp;
-            sp.aip = unmangle(P.Ainv, y);
-            sp.nat = nat;
-            eq4_fast(P.g, P.theta, nat, up, log1pf(-(float)up), sp.est, sp.flags);
-            emit(o.status, csip, report, out_cap, sp);
+        __syncthreads();
+        if ((uint32_t)(tid & ~31) < nt) {
+            const bool ok = (uint32_t)tid < nt;
+            asse_superpoint sp{};
+            if (ok) {
+                const uint32_t y = (uint32_t)(((uint64_t)tuple_at(cur_s, cur_g, t0 + tid)->L << P.u) | j);
+                sp.aip = unmangle(P.Ainv, y);
+                sp.nat = nat_s[tid];
+                eq4_fast(P.g, P.theta, sp.nat, up_s, b_up_s, sp.est, sp.flags);
+            }
+            emit(o.status, csip, report, out_cap, sp, ok);
         }
     }
 }
