@@ -50,17 +50,14 @@ struct asse_pool {
     uint64_t out_cap = 0;
     Status *status = nullptr;
     Status *status_host = nullptr;
-    // asse_close_slice also copies the status and the head of the report to
-    // pinned host memory, so that reading a short report takes one wait
+    // the restore of a close also writes the status and the head of the report
+    // to pinned host memory (status_host, report_host), so that reading a short
+    // report takes one wait, for the close only
     asse_superpoint *report_host = nullptr;
     uint64_t report_host_cap = 0;
     int report_host_valid = 0;
-    cudaEvent_t close_done = nullptr;  // recorded after those copies: a report waits for its close only
-    // the copies of a close's status and report to pinned memory run on their
-    // own stream, after `closed`, so the next batch's ingest does not wait
-    // for them; the next close waits for close_done before it rewrites them
-    cudaStream_t d2h_stream = nullptr;
-    cudaEvent_t closed = nullptr;
+    cudaEvent_t close_done = nullptr;  // recorded after the last close
+    Status *status_read = nullptr;     // pinned, for reading any other status
     // asse_set_timing: events around the scan and the restore of each close
     cudaEvent_t tev[3] = {nullptr, nullptr, nullptr};
     int timing = 0, timed = 0;
@@ -78,7 +75,10 @@ struct asse_pool {
         uint32_t *sa_n = nullptr, *sa_x = nullptr, *sa_mask = nullptr;
         Status *status = nullptr;
         asse_superpoint *csip = nullptr, *report = nullptr;
+        Status *status_host = nullptr;
+        asse_superpoint *report_host = nullptr;
     } win[MAX_WINDOWS - 1];
+    int stream_changed = 0;  // asse_set_stream since the last scan, restore or close
     uint32_t n_windows = 1, sel = 0;  // windows of the last close, the one the readers return
     int scanned = 0, refreshed = 0, restored = 0, ingested = 0;
     uint32_t scan_kp = 0;
@@ -211,13 +211,21 @@ __global__ void init_pool_kernel(uint32_t *pool, uint64_t nwords, uint32_t Wd, u
     }
 }
 
-// Work of the pool's stream that rewrites the status or the report waits
-// until the last close's copies of them (on d2h_stream) have read them.  Not
-// for captured graphs (their closes copy on their own stream in order).
-int wait_close_copies(asse_pool *p)
+// On a stream set since, work that rewrites what the last close wrote waits for
+// that close.
+int wait_last_close(asse_pool *p)
 {
-    CK(p, cudaStreamWaitEvent(p->stream, p->close_done, 0));
+    if (p->stream_changed)
+        CK(p, cudaStreamWaitEvent(p->stream, p->close_done, 0));
+    p->stream_changed = 0;
     return ASSE_OK;
+}
+
+// Where the restore of window m of a close writes for the host.
+HostReport host_report_w(asse_pool *p, uint32_t m)
+{
+    return m == 0 ? HostReport{p->status_host, p->report_host, p->report_host_cap}
+                  : HostReport{p->win[m - 1].status_host, p->win[m - 1].report_host, p->report_host_cap};
 }
 
 int reset_close_state(asse_pool *p)
@@ -239,18 +247,18 @@ int read_list(asse_pool *p, bool reported, asse_superpoint *out, uint64_t cap, u
         return fail(p, ASSE_EINVAL, "NULL argument");
     if (!p->restored)
         return fail(p, ASSE_ESTATE, "no restore since the last scan");
-    const bool early = reported && where != ASSE_DEVICE && p->report_host_valid && p->sel == 0;
+    const bool early = reported && where != ASSE_DEVICE && p->report_host_valid;
+    const HostReport host = host_report_w(p, p->sel);
     if (!early) {
-        CK(p, cudaEventSynchronize(p->close_done));  // no close's copy is still writing status_host
-        CK(p, cudaMemcpyAsync(p->status_host, scan_out_w(p, p->sel).status, sizeof(Status), cudaMemcpyDeviceToHost,
+        CK(p, cudaMemcpyAsync(p->status_read, scan_out_w(p, p->sel).status, sizeof(Status), cudaMemcpyDeviceToHost,
                               p->stream));
         CK(p, cudaStreamSynchronize(p->stream));
     } else {
-        // the close and its copies to pinned memory are done; later work
-        // already queued on the stream (the next batch) keeps running
+        // the close is done; later work already queued on the stream (the
+        // next batch) keeps running
         CK(p, cudaEventSynchronize(p->close_done));
     }
-    const Status st = *p->status_host;
+    const Status st = early ? *host.status : *p->status_read;
     if (st.overflow) {
         *n_out = st.needed;
         char buf[200];
@@ -264,7 +272,7 @@ int read_list(asse_pool *p, bool reported, asse_superpoint *out, uint64_t cap, u
     if (m > 0 && early && m <= p->report_host_cap) {
         if (!out)
             return fail(p, ASSE_EINVAL, "out is NULL");
-        memcpy(out, p->report_host, m * sizeof(asse_superpoint));
+        memcpy(out, host.report, m * sizeof(asse_superpoint));
     } else if (m > 0) {
         if (!out)
             return fail(p, ASSE_EINVAL, "out is NULL");
@@ -298,20 +306,21 @@ void free_all(asse_pool *p)
     cudaFree(p->stage[1]);
     cudaFree(p->q_aips);
     cudaFree(p->q_out);
-    for (auto &w : p->win)
+    for (auto &w : p->win) {
+        if (w.status_host)
+            cudaFreeHost(w.status_host);
         for (void *ptr : {(void *)w.cnt, (void *)w.aat, (void *)w.sa_n, (void *)w.sa_x, (void *)w.sa_mask,
                           (void *)w.status, (void *)w.csip, (void *)w.report})
             cudaFree(ptr);
+    }
     if (p->status_host)
         cudaFreeHost(p->status_host);
+    if (p->status_read)
+        cudaFreeHost(p->status_read);
     if (p->report_host)
         cudaFreeHost(p->report_host);
     if (p->close_done)
         cudaEventDestroy(p->close_done);
-    if (p->closed)
-        cudaEventDestroy(p->closed);
-    if (p->d2h_stream)
-        cudaStreamDestroy(p->d2h_stream);
     for (cudaEvent_t ev : p->tev)
         if (ev)
             cudaEventDestroy(ev);
@@ -343,7 +352,7 @@ int pool_restore_view(asse_pool *p, RestoreView *v)
 
 int pool_fail(asse_pool *p, int code, const std::string &msg) { return fail(p, code, msg); }
 
-int pool_enqueue_close(asse_pool *p, uint32_t kp, bool timed)
+int pool_enqueue_close(asse_pool *p, uint32_t kp, const HostReport &host, bool timed)
 {
     if (int rc = reset_close_state(p))
         return rc;
@@ -358,7 +367,7 @@ int pool_enqueue_close(asse_pool *p, uint32_t kp, bool timed)
     if (timed)
         CK(p, cudaEventRecord(p->tev[1], p->stream));
     CK(p, launch_restore(p->P, scan_out(p), p->scratch, p->cap, p->csip, p->report, p->out_cap, p->stream,
-                         &p->launches, p->ctl));
+                         &p->launches, p->ctl, host));
     if (timed)
         CK(p, cudaEventRecord(p->tev[2], p->stream));
     return ASSE_OK;
@@ -376,10 +385,10 @@ int pool_enqueue_scan(asse_pool *p, uint32_t kp)
     return ASSE_OK;
 }
 
-int pool_enqueue_restore_refresh(asse_pool *p)
+int pool_enqueue_restore_refresh(asse_pool *p, const HostReport &host)
 {
     CK(p, launch_restore(p->P, scan_out(p), p->scratch, p->cap, p->csip, p->report, p->out_cap, p->stream,
-                         &p->launches));
+                         &p->launches, nullptr, host));
     CK(p, launch_refresh(p->P, p->w, p->pool, p->ctl, p->sms, p->stream, &p->launches));
     CK(p, launch_advance_ctl(p->P, p->ctl, p->stream, &p->launches));
     return ASSE_OK;
@@ -424,16 +433,7 @@ int pool_enqueue_ingest(asse_pool *p, const uint32_t *pairs_dev, const unsigned 
     return ASSE_OK;
 }
 
-PoolBuffers pool_buffers(asse_pool *p)
-{
-    PoolBuffers b;
-    b.status = p->status;
-    b.report = p->report;
-    b.out_cap = p->out_cap;
-    b.stream = p->stream;
-    b.cap = p->cap;
-    return b;
-}
+uint32_t pool_restore_cap(const asse_pool *p) { return p->cap; }
 
 // Whether a pool that fits in the L2 cache takes a key table it could do
 // without (key_table AUTO): for plain timestamps and aging counters, whose
@@ -635,6 +635,8 @@ int asse_create(const asse_config *cfg, void *stream, asse_pool **out)
     }
     if (e == cudaSuccess)
         e = cudaMallocHost((void **)&p->status_host, sizeof(Status));
+    if (e == cudaSuccess)
+        e = cudaMallocHost((void **)&p->status_read, sizeof(Status));
     p->report_host_cap = p->out_cap < 4096 ? p->out_cap : 4096;
     if (e == cudaSuccess)
         e = cudaMallocHost((void **)&p->report_host, p->report_host_cap * sizeof(asse_superpoint));
@@ -642,10 +644,6 @@ int asse_create(const asse_config *cfg, void *stream, asse_pool **out)
         e = cudaEventCreateWithFlags(&p->close_done, cudaEventDisableTiming);
     if (e == cudaSuccess)
         e = cudaStreamCreateWithFlags(&p->copy_stream, cudaStreamNonBlocking);
-    if (e == cudaSuccess)
-        e = cudaStreamCreateWithFlags(&p->d2h_stream, cudaStreamNonBlocking);
-    if (e == cudaSuccess)
-        e = cudaEventCreateWithFlags(&p->closed, cudaEventDisableTiming);
     for (int i = 0; i < 2 && e == cudaSuccess; i++) {
         e = cudaEventCreateWithFlags(&p->copied[i], cudaEventDisableTiming);
         if (e == cudaSuccess)
@@ -701,7 +699,7 @@ void asse_destroy(asse_pool *pool)
         return;
     cudaStreamSynchronize(pool->stream);
     cudaStreamSynchronize(pool->copy_stream);
-    cudaStreamSynchronize(pool->d2h_stream);
+    cudaEventSynchronize(pool->close_done);  // of another stream, if it was changed
     free_all(pool);
     delete pool;
 }
@@ -711,6 +709,7 @@ int asse_set_stream(asse_pool *pool, void *stream)
     if (!pool)
         return ASSE_EINVAL;
     pool->stream = (cudaStream_t)stream;
+    pool->stream_changed = 1;
     return ASSE_OK;
 }
 
@@ -763,7 +762,7 @@ int asse_scan(asse_pool *p, uint32_t kp)
         return fail(nullptr, ASSE_EINVAL, "pool is NULL");
     if (int rc = check_kp(p, kp))
         return rc;
-    if (int rc = wait_close_copies(p))
+    if (int rc = wait_last_close(p))
         return rc;
     if (int rc = pool_enqueue_scan(p, kp))
         return rc;
@@ -786,7 +785,7 @@ int asse_restore(asse_pool *p)
     if (!p->scanned)
         return fail(p, ASSE_ESTATE, "restore needs a scan of the open slice");
     p->report_host_valid = 0;
-    if (int rc = wait_close_copies(p))
+    if (int rc = wait_last_close(p))
         return rc;
     CK(p, launch_restore(p->P, scan_out(p), p->scratch, p->cap, p->csip, p->report, p->out_cap, p->stream,
                          &p->launches));
@@ -811,18 +810,13 @@ int asse_close_slice(asse_pool *p, uint32_t kp)
         return fail(nullptr, ASSE_EINVAL, "pool is NULL");
     if (int rc = check_kp(p, kp))
         return rc;
-    if (int rc = wait_close_copies(p))
+    if (int rc = wait_last_close(p))
         return rc;
-    if (int rc = pool_enqueue_close(p, kp, p->timing != 0))
+    if (int rc = pool_enqueue_close(p, kp, host_report_w(p, 0), p->timing != 0))
         return rc;
     pool_after_close(p, kp);
     p->timed = p->timing;
-    CK(p, cudaEventRecord(p->closed, p->stream));
-    CK(p, cudaStreamWaitEvent(p->d2h_stream, p->closed, 0));
-    CK(p, cudaMemcpyAsync(p->status_host, p->status, sizeof(Status), cudaMemcpyDeviceToHost, p->d2h_stream));
-    CK(p, cudaMemcpyAsync(p->report_host, p->report, p->report_host_cap * sizeof(asse_superpoint),
-                          cudaMemcpyDeviceToHost, p->d2h_stream));
-    CK(p, cudaEventRecord(p->close_done, p->d2h_stream));
+    CK(p, cudaEventRecord(p->close_done, p->stream));
     p->report_host_valid = 1;
     return ASSE_OK;
 }
@@ -856,6 +850,11 @@ int asse_close_slice_multi(asse_pool *p, const uint32_t *kps, uint32_t n_windows
         alloc((void **)&w.status, sizeof(Status));
         alloc((void **)&w.csip, p->out_cap * sizeof(asse_superpoint));
         alloc((void **)&w.report, p->out_cap * sizeof(asse_superpoint));
+        // the status, then the head of the report
+        if (e == cudaSuccess)
+            e = cudaMallocHost((void **)&w.status_host, 256 + p->report_host_cap * sizeof(asse_superpoint));
+        if (e == cudaSuccess)
+            w.report_host = reinterpret_cast<asse_superpoint *>(reinterpret_cast<char *>(w.status_host) + 256);
         if (e != cudaSuccess) {
             cudaGetLastError();
             for (void *ptr : {(void *)w.cnt, (void *)w.aat, (void *)w.sa_n, (void *)w.sa_x, (void *)w.sa_mask,
@@ -866,7 +865,7 @@ int asse_close_slice_multi(asse_pool *p, const uint32_t *kps, uint32_t n_windows
                                                   : cuda_fail(p, e, "window outputs");
         }
     }
-    if (int rc = wait_close_copies(p))
+    if (int rc = wait_last_close(p))
         return rc;
     ScanWindows W{};
     W.n = n_windows;
@@ -883,17 +882,20 @@ int asse_close_slice_multi(asse_pool *p, const uint32_t *kps, uint32_t n_windows
                                    &p->launches));
         for (uint32_t m = 0; m < n_windows; m++)
             CK(p, launch_restore(p->P, W.o[m], p->scratch, p->cap, list_w(p, m, false), list_w(p, m, true),
-                                 p->out_cap, p->stream, &p->launches));
+                                 p->out_cap, p->stream, &p->launches, nullptr, host_report_w(p, m)));
         CK(p, launch_refresh(p->P, p->w, p->pool, p->ctl, p->sms, p->stream, &p->launches));
         CK(p, launch_advance_ctl(p->P, p->ctl, p->stream, &p->launches));
     } else {
         CK(p, launch_scan_windows(p->P, p->w, p->pool, W, p->ctl, p->sms, p->stream, &p->launches));
         for (uint32_t m = 0; m < n_windows; m++)
             CK(p, launch_restore(p->P, W.o[m], p->scratch, p->cap, list_w(p, m, false), list_w(p, m, true),
-                                 p->out_cap, p->stream, &p->launches, m + 1 == n_windows ? p->ctl : nullptr));
+                                 p->out_cap, p->stream, &p->launches, m + 1 == n_windows ? p->ctl : nullptr,
+                                 host_report_w(p, m)));
     }
     pool_after_close(p, kps[0]);
     p->n_windows = n_windows;
+    CK(p, cudaEventRecord(p->close_done, p->stream));
+    p->report_host_valid = 1;
     return ASSE_OK;
 }
 

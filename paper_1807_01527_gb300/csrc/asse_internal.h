@@ -136,7 +136,8 @@ struct Status {
     unsigned long long n_report;  // candidates with estimate >= theta
     unsigned long long needed;    // tuples the overflowing join level needed
     unsigned int overflow;        // a frame exceeded the restore capacity
-    unsigned int pad[5];
+    unsigned int done;            // restore blocks that have finished
+    unsigned int pad[4];
 };
 
 // A partial or complete column tuple of the restore join.
@@ -272,11 +273,18 @@ cudaError_t launch_scan_windows(const Params &P, uint32_t w, uint32_t *pool, con
                                 const SliceCtl *ctl, int sms, cudaStream_t s, uint64_t *launches);
 cudaError_t launch_refresh(const Params &P, uint32_t w, uint32_t *pool, const SliceCtl *ctl, int sms, cudaStream_t s,
                            uint64_t *launches);
+// Pinned host memory that the restore also writes the status and the first
+// cap reported records to (report null: it does not).
+struct HostReport {
+    Status *status = nullptr;
+    asse_superpoint *report = nullptr;
+    uint64_t cap = 0;
+};
 // advance (may be null): the restore also opens the next slice, as
 // launch_advance_ctl would (the fused close saves that launch).
 cudaError_t launch_restore(const Params &P, const ScanOut &o, Tuple *scratch, uint32_t cap, asse_superpoint *csip,
                            asse_superpoint *report, uint64_t out_cap, cudaStream_t s, uint64_t *launches,
-                           SliceCtl *advance = nullptr);
+                           SliceCtl *advance = nullptr, const HostReport &host = HostReport());
 cudaError_t launch_estimate(const Params &P, uint32_t w, const uint32_t *pool, uint32_t c0, uint32_t kp,
                             const unsigned long long *aat, const uint32_t *aips, uint64_t n, asse_superpoint *out,
                             int sms, cudaStream_t s, uint64_t *launches);
@@ -341,23 +349,16 @@ int pool_fail(asse_pool *p, int code, const std::string &msg);
 // which captures them into CUDA graphs: enqueue the device work of a close
 // (no host bookkeeping), do the host bookkeeping of one close, and enqueue an
 // ingest whose pair count is read from device memory.
-int pool_enqueue_close(asse_pool *p, uint32_t kp, bool timed = false);
+int pool_enqueue_close(asse_pool *p, uint32_t kp, const HostReport &host, bool timed = false);
 // The same close in three parts, for a close with learned inference between
 // the scan and the refresh (the refresh changes the state the features read):
 // the scan alone, then (after the caller's work) the restore, the refresh and
 // the opening of the next slice.
 int pool_enqueue_scan(asse_pool *p, uint32_t kp);
-int pool_enqueue_restore_refresh(asse_pool *p);
+int pool_enqueue_restore_refresh(asse_pool *p, const HostReport &host);
 void pool_after_close(asse_pool *p, uint32_t kp);
 int pool_enqueue_ingest(asse_pool *p, const uint32_t *pairs_dev, const unsigned long long *n_dev);
-struct PoolBuffers {
-    Status *status;
-    asse_superpoint *report;
-    uint64_t out_cap;
-    cudaStream_t stream;
-    uint32_t cap;
-};
-PoolBuffers pool_buffers(asse_pool *p);
+uint32_t pool_restore_cap(const asse_pool *p);
 uint64_t pool_device_bytes(const asse_config *cfg);
 // Whether key_table AUTO of cfg keeps a key table because the pool is larger
 // than the current device's L2 cache.

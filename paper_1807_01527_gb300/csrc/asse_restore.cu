@@ -87,7 +87,7 @@ __device__ __forceinline__ double frame_up(const Params &P, const unsigned long 
 // The candidates of a warp (one per lane, if ok) join CSIP, those that reach
 // theta the report too: one atomic per list for the warp.
 __device__ __forceinline__ void emit(Status *st, asse_superpoint *csip, asse_superpoint *report, uint64_t out_cap,
-                                     const asse_superpoint &sp, bool ok)
+                                     const HostReport &host, const asse_superpoint &sp, bool ok)
 {
     const unsigned lane = threadIdx.x & 31, lt = (1u << lane) - 1u;
     const bool rep = ok && (sp.flags & ASSE_SP_REPORTED) != 0;
@@ -103,6 +103,8 @@ __device__ __forceinline__ void emit(Status *st, asse_superpoint *csip, asse_sup
         csip[p] = sp;
     if (rep && p2 < out_cap)
         report[p2] = sp;
+    if (rep && p2 < host.cap)
+        *reinterpret_cast<uint4 *>(host.report + p2) = make_uint4(sp.aip, sp.nat, __float_as_uint(sp.est), sp.flags);
 }
 
 constexpr int RESTORE_THREADS = 512;
@@ -122,13 +124,10 @@ __device__ __forceinline__ Tuple *tuple_at(Tuple *sm, Tuple *gl, uint32_t a)
     return a < RESTORE_SMEM_TUPLES ? sm + a : gl + a;
 }
 
-__global__ void __launch_bounds__(RESTORE_THREADS) restore_kernel(Params P, ScanOut o, Tuple *scratch, uint32_t cap,
-                                                                  asse_superpoint *csip, asse_superpoint *report,
-                                                                  uint64_t out_cap, SliceCtl *advance)
+// The restore of frame blockIdx.x.
+__device__ void restore_frame(const Params &P, const ScanOut &o, Tuple *scratch, uint32_t cap, asse_superpoint *csip,
+                              asse_superpoint *report, uint64_t out_cap, const HostReport &host)
 {
-    // the scan of this close has read the slice state; open the next slice
-    if (advance != nullptr && blockIdx.x == 0)
-        open_next_slice(P, advance);
     __shared__ uint32_t n_sa[8];
     __shared__ double p_row[8];  // |AAT(k',i,j)| / (g 2^c) of each row (Sec. 4.3)
     __shared__ uint32_t n_next;
@@ -295,7 +294,35 @@ __global__ void __launch_bounds__(RESTORE_THREADS) restore_kernel(Params P, Scan
                 sp.nat = nat_s[tid];
                 eq4_fast(P.g, P.theta, sp.nat, up_s, b_up_s, sp.est, sp.flags);
             }
-            emit(o.status, csip, report, out_cap, sp, ok);
+            emit(o.status, csip, report, out_cap, host, sp, ok);
+        }
+    }
+}
+
+// One block per frame.  With a host report, the reported records are also
+// written to pinned host memory as they are found, and the last block to finish
+// writes the status there: a report then waits for this kernel alone.  Copies
+// of both on a stream of their own after the restore came 13 us after its end.
+__global__ void __launch_bounds__(RESTORE_THREADS) restore_kernel(Params P, ScanOut o, Tuple *scratch, uint32_t cap,
+                                                                  asse_superpoint *csip, asse_superpoint *report,
+                                                                  uint64_t out_cap, SliceCtl *advance, HostReport host)
+{
+    // the scan of this close has read the slice state; open the next slice
+    if (advance != nullptr && blockIdx.x == 0)
+        open_next_slice(P, advance);
+    restore_frame(P, o, scratch, cap, csip, report, out_cap, host);
+    if (host.status == nullptr)
+        return;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        __threadfence();  // this block's counts before its own
+        if (atomicAdd(&o.status->done, 1u) + 1 == gridDim.x) {
+            __threadfence();
+            volatile Status *st = o.status;
+            host.status->n_csip = st->n_csip;
+            host.status->n_report = st->n_report;
+            host.status->needed = st->needed;
+            host.status->overflow = st->overflow;
         }
     }
 }
@@ -395,10 +422,10 @@ __global__ void __launch_bounds__(ESTIMATE_THREADS) estimate_kernel(Params P, co
 
 cudaError_t launch_restore(const Params &P, const ScanOut &o, Tuple *scratch, uint32_t cap, asse_superpoint *csip,
                            asse_superpoint *report, uint64_t out_cap, cudaStream_t s, uint64_t *launches,
-                           SliceCtl *advance)
+                           SliceCtl *advance, const HostReport &host)
 {
     *launches += 1;
-    restore_kernel<<<P.nf, RESTORE_THREADS, 0, s>>>(P, o, scratch, cap, csip, report, out_cap, advance);
+    restore_kernel<<<P.nf, RESTORE_THREADS, 0, s>>>(P, o, scratch, cap, csip, report, out_cap, advance, host);
     return cudaGetLastError();
 }
 

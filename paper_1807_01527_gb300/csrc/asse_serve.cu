@@ -119,10 +119,11 @@ cudaError_t capture(cudaStream_t s, cudaGraphExec_t *out, Fn &&enqueue, int *rc)
 // Capture the close of one report slot: the fused close (scan with the
 // refresh, restore, next slice) or, with a model attached, the scan, the
 // learned inference of every ATV, then the restore, the refresh and the next
-// slice; then the copies of the status and the report (and the fallback
-// count) to the slot's pinned memory.
-cudaError_t capture_close(SStream *st, Slot &sl, const PoolBuffers &pb, int *rc)
+// slice, and the copy of the fallback count; the restore writes the status and
+// the report to the slot's pinned memory.
+cudaError_t capture_close(SStream *st, Slot &sl, int *rc)
 {
+    const HostReport host{sl.status_host, sl.report_host, st->rcap};
     return capture(st->s, &sl.graph,
                    [&]() {
                        if (st->mlp) {
@@ -133,19 +134,14 @@ cudaError_t capture_close(SStream *st, Slot &sl, const PoolBuffers &pb, int *rc)
                            if (int r = mlp_enqueue_learned(st->mlp, v, st->max_log_n, st->x, sl.est, sl.nfb_dev,
                                                            &why))
                                return pool_fail(st->pool, r, "learned inference: " + why);
-                           if (int r = pool_enqueue_restore_refresh(st->pool))
+                           if (int r = pool_enqueue_restore_refresh(st->pool, host))
                                return r;
                            if (cudaMemcpyAsync(sl.nfb_host, sl.nfb_dev, sizeof(uint32_t), cudaMemcpyDeviceToHost,
                                                st->s) != cudaSuccess)
                                return (int)ASSE_ECUDA;
-                       } else if (int r = pool_enqueue_close(st->pool, st->kp)) {
+                       } else if (int r = pool_enqueue_close(st->pool, st->kp, host)) {
                            return r;
                        }
-                       if (cudaMemcpyAsync(sl.status_host, pb.status, sizeof(Status), cudaMemcpyDeviceToHost,
-                                           st->s) != cudaSuccess ||
-                           cudaMemcpyAsync(sl.report_host, pb.report, st->rcap * sizeof(asse_superpoint),
-                                           cudaMemcpyDeviceToHost, st->s) != cudaSuccess)
-                           return (int)ASSE_ECUDA;
                        return (int)ASSE_OK;
                    },
                    rc);
@@ -250,8 +246,7 @@ int asse_server_open(asse_server *srv, const asse_config *cfg, uint32_t kp, uint
         e = cudaMalloc((void **)&st->staging, max_batch * 8);
     if (e == cudaSuccess)
         e = cudaMalloc((void **)&st->n_dev, sizeof(unsigned long long));
-    const PoolBuffers pb = e == cudaSuccess ? pool_buffers(st->pool) : PoolBuffers{};
-    st->rcap = pb.cap;
+    st->rcap = e == cudaSuccess ? pool_restore_cap(st->pool) : 0;
     if (e == cudaSuccess)
         e = capture(st->s, &st->ingest, [&]() { return pool_enqueue_ingest(st->pool, st->staging, st->n_dev); },
                     &rc);
@@ -268,7 +263,7 @@ int asse_server_open(asse_server *srv, const asse_config *cfg, uint32_t kp, uint
         if (e == cudaSuccess)
             e = cudaEventCreate(&sl.done);
         if (e == cudaSuccess)
-            e = capture_close(st, sl, pb, &rc);
+            e = capture_close(st, sl, &rc);
     }
     if (e == cudaSuccess && rc == ASSE_OK)
         e = cudaStreamSynchronize(st->s);
@@ -421,7 +416,6 @@ int asse_server_attach_model(asse_server *srv, uint32_t id, asse_mlp *mlp, float
     }
     st->mlp = mlp;
     st->max_log_n = max_log_n;
-    const PoolBuffers pb = pool_buffers(st->pool);
     int rc = ASSE_OK;
     for (Slot &sl : st->ring) {
         if (e != cudaSuccess || rc != ASSE_OK)
@@ -430,7 +424,7 @@ int asse_server_attach_model(asse_server *srv, uint32_t id, asse_mlp *mlp, float
             cudaGraphExecDestroy(sl.graph);
             sl.graph = nullptr;
         }
-        e = capture_close(st, sl, pb, &rc);
+        e = capture_close(st, sl, &rc);
     }
     if (e == cudaSuccess && rc == ASSE_OK)
         e = cudaStreamSynchronize(st->s);
