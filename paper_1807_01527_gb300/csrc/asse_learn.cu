@@ -685,8 +685,7 @@ int asse_synth_states(const asse_synth_cfg *cfg, uint64_t first, uint64_t n, uin
     // ATVs of more than 933 words (g above 3,712 in byte-wide fields) are refused
     if (P.Wd > 933)
         return ASSE_ECUDA;
-    // a feature row counts the first 32 FEAT_MAXM words of an ATV, as the pool's kernels do
-    const uint32_t visible = 32 * FEAT_MAXM * Fw;
+    const uint32_t visible = 512 * Fw;  // a feature row counts the first 512 words of an ATV, all a pool's can have
     int dev = 0, sms = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
