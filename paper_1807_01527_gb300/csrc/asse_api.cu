@@ -70,11 +70,13 @@ struct asse_pool {
     // outputs of windows 1 .. MAX_WINDOWS-1 of a multi-window close (window 0
     // uses the buffers above), allocated on first use
     struct Win {
+        unsigned char *block = nullptr;  // holds all of the device ones
         uint16_t *cnt = nullptr;
         unsigned long long *aat = nullptr;
         uint32_t *sa_n = nullptr, *sa_x = nullptr, *sa_mask = nullptr;
         Status *status = nullptr;
         asse_superpoint *csip = nullptr, *report = nullptr;
+        Tuple *scratch = nullptr;
         Status *status_host = nullptr;
         asse_superpoint *report_host = nullptr;
     } win[MAX_WINDOWS - 1];
@@ -230,7 +232,10 @@ HostReport host_report_w(asse_pool *p, uint32_t m)
 
 int reset_close_state(asse_pool *p)
 {
-    CK(p, launch_reset(p->aat, p->sa_n, p->cfg.r * p->P.nf, p->status, p->stream, &p->launches));
+    ScanWindows W{};
+    W.n = 1;
+    W.o[0] = scan_out(p);
+    CK(p, launch_reset(W, p->cfg.r * p->P.nf, p->stream, &p->launches));
     return ASSE_OK;
 }
 
@@ -309,9 +314,7 @@ void free_all(asse_pool *p)
     for (auto &w : p->win) {
         if (w.status_host)
             cudaFreeHost(w.status_host);
-        for (void *ptr : {(void *)w.cnt, (void *)w.aat, (void *)w.sa_n, (void *)w.sa_x, (void *)w.sa_mask,
-                          (void *)w.status, (void *)w.csip, (void *)w.report})
-            cudaFree(ptr);
+        cudaFree(w.block);
     }
     if (p->status_host)
         cudaFreeHost(p->status_host);
@@ -837,60 +840,65 @@ int asse_close_slice_multi(asse_pool *p, const uint32_t *kps, uint32_t n_windows
         asse_pool::Win &w = p->win[m - 1];
         if (w.cnt)
             continue;
-        cudaError_t e = cudaSuccess;
-        auto alloc = [&](void **ptr, size_t bytes) {
-            if (e == cudaSuccess)
-                e = cudaMalloc(ptr, bytes);
+        // one allocation, in 256-byte aligned parts
+        size_t bytes = 0;
+        auto part = [&](size_t n) {
+            const size_t at = bytes;
+            bytes += (n + 255) / 256 * 256;
+            return at;
         };
-        alloc((void **)&w.cnt, n_atv * sizeof(uint16_t));
-        alloc((void **)&w.aat, nseg * sizeof(unsigned long long));
-        alloc((void **)&w.sa_n, nseg * sizeof(uint32_t));
-        alloc((void **)&w.sa_x, n_atv * sizeof(uint32_t));
-        alloc((void **)&w.sa_mask, n_atv * p->P.mw * sizeof(uint32_t));
-        alloc((void **)&w.status, sizeof(Status));
-        alloc((void **)&w.csip, p->out_cap * sizeof(asse_superpoint));
-        alloc((void **)&w.report, p->out_cap * sizeof(asse_superpoint));
+        const size_t cnt = part(n_atv * sizeof(uint16_t)), aat = part(nseg * sizeof(unsigned long long)),
+                     sa_n = part(nseg * sizeof(uint32_t)), sa_x = part(n_atv * sizeof(uint32_t)),
+                     sa_mask = part(n_atv * p->P.mw * sizeof(uint32_t)), status = part(sizeof(Status)),
+                     csip = part(p->out_cap * sizeof(asse_superpoint)),
+                     report = part(p->out_cap * sizeof(asse_superpoint)),
+                     scratch = part((size_t)p->P.nf * 2 * p->cap * sizeof(Tuple));
+        cudaError_t e = cudaMalloc((void **)&w.block, bytes);
         // the status, then the head of the report
         if (e == cudaSuccess)
             e = cudaMallocHost((void **)&w.status_host, 256 + p->report_host_cap * sizeof(asse_superpoint));
-        if (e == cudaSuccess)
-            w.report_host = reinterpret_cast<asse_superpoint *>(reinterpret_cast<char *>(w.status_host) + 256);
         if (e != cudaSuccess) {
             cudaGetLastError();
-            for (void *ptr : {(void *)w.cnt, (void *)w.aat, (void *)w.sa_n, (void *)w.sa_x, (void *)w.sa_mask,
-                              (void *)w.status, (void *)w.csip, (void *)w.report})
-                cudaFree(ptr);
+            cudaFree(w.block);
             w = asse_pool::Win();
             return e == cudaErrorMemoryAllocation ? fail(p, ASSE_ENOMEM, "window outputs: device allocation failed")
                                                   : cuda_fail(p, e, "window outputs");
         }
+        w.report_host = reinterpret_cast<asse_superpoint *>(reinterpret_cast<char *>(w.status_host) + 256);
+        w.cnt = reinterpret_cast<uint16_t *>(w.block + cnt);
+        w.aat = reinterpret_cast<unsigned long long *>(w.block + aat);
+        w.sa_n = reinterpret_cast<uint32_t *>(w.block + sa_n);
+        w.sa_x = reinterpret_cast<uint32_t *>(w.block + sa_x);
+        w.sa_mask = reinterpret_cast<uint32_t *>(w.block + sa_mask);
+        w.status = reinterpret_cast<Status *>(w.block + status);
+        w.csip = reinterpret_cast<asse_superpoint *>(w.block + csip);
+        w.report = reinterpret_cast<asse_superpoint *>(w.block + report);
+        w.scratch = reinterpret_cast<Tuple *>(w.block + scratch);
     }
     if (int rc = wait_last_close(p))
         return rc;
     ScanWindows W{};
+    RestoreWindows out{};
     W.n = n_windows;
     for (uint32_t m = 0; m < n_windows; m++) {
         W.kp[m] = kps[m];
         W.o[m] = scan_out_w(p, m);
-        CK(p, launch_reset(W.o[m].aat, W.o[m].sa_n, p->cfg.r * p->P.nf, W.o[m].status, p->stream, &p->launches));
+        out.w[m] = RestoreOut{m == 0 ? p->scratch : p->win[m - 1].scratch, list_w(p, m, false), list_w(p, m, true),
+                              host_report_w(p, m)};
     }
+    CK(p, launch_reset(W, p->cfg.r * p->P.nf, p->stream, &p->launches));
     if (p->P.hist) {
-        // one count pass per window over the slice counts, then the restores,
+        // one count pass per window over the slice counts, then the restore,
         // the refresh (with the zeroing of the next slice's counts) and the next slice
         for (uint32_t m = 0; m < n_windows; m++)
             CK(p, launch_hist_scan(p->P, p->w, p->pool, kps[m], false, p->ctl, W.o[m], p->sms, p->stream,
                                    &p->launches));
-        for (uint32_t m = 0; m < n_windows; m++)
-            CK(p, launch_restore(p->P, W.o[m], p->scratch, p->cap, list_w(p, m, false), list_w(p, m, true),
-                                 p->out_cap, p->stream, &p->launches, nullptr, host_report_w(p, m)));
+        CK(p, launch_restores(p->P, W, p->cap, out, p->out_cap, p->stream, &p->launches));
         CK(p, launch_refresh(p->P, p->w, p->pool, p->ctl, p->sms, p->stream, &p->launches));
         CK(p, launch_advance_ctl(p->P, p->ctl, p->stream, &p->launches));
     } else {
         CK(p, launch_scan_windows(p->P, p->w, p->pool, W, p->ctl, p->sms, p->stream, &p->launches));
-        for (uint32_t m = 0; m < n_windows; m++)
-            CK(p, launch_restore(p->P, W.o[m], p->scratch, p->cap, list_w(p, m, false), list_w(p, m, true),
-                                 p->out_cap, p->stream, &p->launches, m + 1 == n_windows ? p->ctl : nullptr,
-                                 host_report_w(p, m)));
+        CK(p, launch_restores(p->P, W, p->cap, out, p->out_cap, p->stream, &p->launches, p->ctl));
     }
     pool_after_close(p, kps[0]);
     p->n_windows = n_windows;

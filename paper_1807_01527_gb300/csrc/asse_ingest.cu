@@ -470,14 +470,15 @@ __global__ void advance_ctl_kernel(Params P, SliceCtl *ctl)
     open_next_slice(P, ctl);
 }
 
-__global__ void reset_kernel(unsigned long long *aat, uint32_t *sa_n, uint32_t nseg, Status *status)
+__global__ void reset_kernel(const __grid_constant__ ScanWindows W, uint32_t nseg)
 {
+    const ScanOut o = W.o[blockIdx.y];
     for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < nseg; i += gridDim.x * blockDim.x) {
-        aat[i] = 0;
-        sa_n[i] = 0;
+        o.aat[i] = 0;
+        o.sa_n[i] = 0;
     }
     if (blockIdx.x == 0 && threadIdx.x == 0)
-        *status = Status{};
+        *o.status = Status{};
 }
 
 }  // namespace
@@ -489,12 +490,10 @@ cudaError_t launch_advance_ctl(const Params &P, SliceCtl *ctl, cudaStream_t s, u
     return cudaGetLastError();
 }
 
-// Zero the scan outputs that are accumulated with atomics, and the status.
-cudaError_t launch_reset(unsigned long long *aat, uint32_t *sa_n, uint32_t nseg, Status *status, cudaStream_t s,
-                         uint64_t *launches)
+cudaError_t launch_reset(const ScanWindows &W, uint32_t nseg, cudaStream_t s, uint64_t *launches)
 {
     *launches += 1;
-    reset_kernel<<<(nseg + 255) / 256 < 1 ? 1 : (nseg + 255) / 256, 256, 0, s>>>(aat, sa_n, nseg, status);
+    reset_kernel<<<dim3((nseg + 255) / 256 < 1 ? 1 : (nseg + 255) / 256, W.n), 256, 0, s>>>(W, nseg);
     return cudaGetLastError();
 }
 

@@ -257,8 +257,6 @@ cudaError_t launch_ingest(const Params &P, uint32_t w, uint32_t *pool, const uin
                           uint64_t *launches);
 // Open the next slice on the device: ctl = slice_ctl(ctl->t + 1).
 cudaError_t launch_advance_ctl(const Params &P, SliceCtl *ctl, cudaStream_t s, uint64_t *launches);
-cudaError_t launch_reset(unsigned long long *aat, uint32_t *sa_n, uint32_t nseg, Status *status, cudaStream_t s,
-                         uint64_t *launches);
 cudaError_t launch_scan(const Params &P, uint32_t w, uint32_t *pool, uint32_t kp, bool fuse, const SliceCtl *ctl,
                         const ScanOut &o, int sms, cudaStream_t s, uint64_t *launches);
 // Several windows k' (Sec. 3: the same ATs answer every k' <= k) counted in
@@ -273,6 +271,8 @@ cudaError_t launch_scan_windows(const Params &P, uint32_t w, uint32_t *pool, con
                                 const SliceCtl *ctl, int sms, cudaStream_t s, uint64_t *launches);
 cudaError_t launch_refresh(const Params &P, uint32_t w, uint32_t *pool, const SliceCtl *ctl, int sms, cudaStream_t s,
                            uint64_t *launches);
+// Zero what the scan of every window of W accumulates with atomics, and its status.
+cudaError_t launch_reset(const ScanWindows &W, uint32_t nseg, cudaStream_t s, uint64_t *launches);
 // Pinned host memory that the restore also writes the status and the first
 // cap reported records to (report null: it does not).
 struct HostReport {
@@ -280,8 +280,22 @@ struct HostReport {
     asse_superpoint *report = nullptr;
     uint64_t cap = 0;
 };
-// advance (may be null): the restore also opens the next slice, as
-// launch_advance_ctl would (the fused close saves that launch).
+// What the restore of one window writes: the join's scratch (2^u frames x 2
+// levels x cap tuples), the lists, and the host's copy.
+struct RestoreOut {
+    Tuple *scratch;
+    asse_superpoint *csip, *report;
+    HostReport host;
+};
+struct RestoreWindows {
+    RestoreOut w[MAX_WINDOWS];
+};
+// One launch for every window of W.  advance (may be null): the restore also
+// opens the next slice, as launch_advance_ctl would (the fused close saves that
+// launch).
+cudaError_t launch_restores(const Params &P, const ScanWindows &W, uint32_t cap, const RestoreWindows &out,
+                            uint64_t out_cap, cudaStream_t s, uint64_t *launches, SliceCtl *advance = nullptr);
+// The restore of one window.
 cudaError_t launch_restore(const Params &P, const ScanOut &o, Tuple *scratch, uint32_t cap, asse_superpoint *csip,
                            asse_superpoint *report, uint64_t out_cap, cudaStream_t s, uint64_t *launches,
                            SliceCtl *advance = nullptr, const HostReport &host = HostReport());

@@ -299,18 +299,22 @@ __device__ void restore_frame(const Params &P, const ScanOut &o, Tuple *scratch,
     }
 }
 
-// One block per frame.  With a host report, the reported records are also
+// One block per frame and window.  With a host report, the reported records are also
 // written to pinned host memory as they are found, and the last block to finish
 // writes the status there: a report then waits for this kernel alone.  Copies
 // of both on a stream of their own after the restore came 13 us after its end.
-__global__ void __launch_bounds__(RESTORE_THREADS) restore_kernel(Params P, ScanOut o, Tuple *scratch, uint32_t cap,
-                                                                  asse_superpoint *csip, asse_superpoint *report,
-                                                                  uint64_t out_cap, SliceCtl *advance, HostReport host)
+__global__ void __launch_bounds__(RESTORE_THREADS) restore_kernel(Params P, const __grid_constant__ ScanWindows W,
+                                                                  uint32_t cap,
+                                                                  const __grid_constant__ RestoreWindows out,
+                                                                  uint64_t out_cap, SliceCtl *advance)
 {
     // the scan of this close has read the slice state; open the next slice
-    if (advance != nullptr && blockIdx.x == 0)
+    if (advance != nullptr && blockIdx.x == 0 && blockIdx.y == 0)
         open_next_slice(P, advance);
-    restore_frame(P, o, scratch, cap, csip, report, out_cap, host);
+    const ScanOut o = W.o[blockIdx.y];
+    const RestoreOut ro = out.w[blockIdx.y];
+    const HostReport host = ro.host;
+    restore_frame(P, o, ro.scratch, cap, ro.csip, ro.report, out_cap, host);
     if (host.status == nullptr)
         return;
     __syncthreads();
@@ -420,13 +424,24 @@ __global__ void __launch_bounds__(ESTIMATE_THREADS) estimate_kernel(Params P, co
 
 }  // namespace
 
+cudaError_t launch_restores(const Params &P, const ScanWindows &W, uint32_t cap, const RestoreWindows &out,
+                            uint64_t out_cap, cudaStream_t s, uint64_t *launches, SliceCtl *advance)
+{
+    *launches += 1;
+    restore_kernel<<<dim3(P.nf, W.n), RESTORE_THREADS, 0, s>>>(P, W, cap, out, out_cap, advance);
+    return cudaGetLastError();
+}
+
 cudaError_t launch_restore(const Params &P, const ScanOut &o, Tuple *scratch, uint32_t cap, asse_superpoint *csip,
                            asse_superpoint *report, uint64_t out_cap, cudaStream_t s, uint64_t *launches,
                            SliceCtl *advance, const HostReport &host)
 {
-    *launches += 1;
-    restore_kernel<<<P.nf, RESTORE_THREADS, 0, s>>>(P, o, scratch, cap, csip, report, out_cap, advance, host);
-    return cudaGetLastError();
+    ScanWindows W{};
+    W.n = 1;
+    W.o[0] = o;
+    RestoreWindows out{};
+    out.w[0] = RestoreOut{scratch, csip, report, host};
+    return launch_restores(P, W, cap, out, out_cap, s, launches, advance);
 }
 
 cudaError_t launch_estimate(const Params &P, uint32_t w, const uint32_t *pool, uint32_t c0, uint32_t kp,
