@@ -173,4 +173,30 @@ int resident_blocks(K kernel, int threads, size_t smem)
     return n;
 }
 
+// Programmatic dependent launch: a kernel launched by launch_dependent may
+// start once every block of the kernel before it on the stream has called
+// let_next_start (or ended), and calls wait_for_last before it touches anything
+// that kernel, or an earlier one, reads or writes: its launch and set-up then
+// overlap that kernel's end.  Every block of such a kernel calls wait_for_last,
+// so that one kernel's wait covers all before it.
+__device__ __forceinline__ void let_next_start() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void wait_for_last() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
+template <typename... KArgs, typename... Args>
+cudaError_t launch_dependent(void (*kernel)(KArgs...), dim3 grid, unsigned threads, size_t smem, cudaStream_t s,
+                             Args &&...args)
+{
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t lc{};
+    lc.gridDim = grid;
+    lc.blockDim = dim3(threads);
+    lc.dynamicSmemBytes = smem;
+    lc.stream = s;
+    lc.attrs = attr;
+    lc.numAttrs = 1;
+    return cudaLaunchKernelEx(&lc, kernel, static_cast<KArgs>(args)...);
+}
+
 }  // namespace asse

@@ -87,6 +87,7 @@ __global__ void __launch_bounds__(HIST_THREADS) hist_scan_kernel(Params P, uint3
             rdesc[q] = refresh_desc<WB>(P, q, R.c0n);
     }
     __syncthreads();
+    wait_for_last();
     uint32_t *my_mask = maskbuf + warp * P.mw;
     // the refreshed words as up to four slots when the (at most two) ranges
     // hold at most four words together
@@ -241,6 +242,7 @@ __global__ void __launch_bounds__(HIST_THREADS) hist_scan_kernel(Params P, uint3
             store_counts<V>(P.hist + (uint64_t)R.c0n * total_atv + a0, zero);
         }
     }
+    let_next_start();
 }
 
 // The slice counts of a pool counted from its words (after asse_load): every
@@ -299,9 +301,8 @@ cudaError_t launch_hist_scan(const Params &P, uint32_t w, uint32_t *pool, uint32
         const uint32_t per = v8 ? 8 : 1;
         const uint64_t want = (total / per + HIST_THREADS - 1) / HIST_THREADS;
         const uint64_t full = (uint64_t)sms * resident_blocks(kern, HIST_THREADS, smem);
-        kern<<<(unsigned)(want < full ? (want < 1 ? 1 : want) : full), HIST_THREADS, smem, s>>>(P, pool, kp, ctl, o,
-                                                                                           total);
-        return cudaGetLastError();
+        return launch_dependent(kern, dim3((unsigned)(want < full ? (want < 1 ? 1 : want) : full)), HIST_THREADS, smem, s,
+                                P, pool, kp, ctl, o, total);
     });
 }
 

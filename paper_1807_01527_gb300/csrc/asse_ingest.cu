@@ -404,6 +404,7 @@ __global__ void __launch_bounds__(INGEST_THREADS, INGEST_BLOCKS_PER_SM)
     // no CTA leaves while another may still read its table
     if constexpr (CLUSTER)
         cooperative_groups::this_cluster().sync();
+    let_next_start();
 }
 
 }  // namespace
@@ -472,6 +473,10 @@ __global__ void advance_ctl_kernel(Params P, SliceCtl *ctl)
 
 __global__ void reset_kernel(const __grid_constant__ ScanWindows W, uint32_t nseg)
 {
+    // the scan may start its set-up, which reads the slice state, only once
+    // what wrote that is over
+    wait_for_last();
+    let_next_start();
     const ScanOut o = W.o[blockIdx.y];
     for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < nseg; i += gridDim.x * blockDim.x) {
         o.aat[i] = 0;
@@ -493,8 +498,7 @@ cudaError_t launch_advance_ctl(const Params &P, SliceCtl *ctl, cudaStream_t s, u
 cudaError_t launch_reset(const ScanWindows &W, uint32_t nseg, cudaStream_t s, uint64_t *launches)
 {
     *launches += 1;
-    reset_kernel<<<dim3((nseg + 255) / 256 < 1 ? 1 : (nseg + 255) / 256, W.n), 256, 0, s>>>(W, nseg);
-    return cudaGetLastError();
+    return launch_dependent(reset_kernel, dim3((nseg + 255) / 256 < 1 ? 1 : (nseg + 255) / 256, W.n), 256, 0, s, W, nseg);
 }
 
 }  // namespace asse

@@ -283,6 +283,8 @@ __global__ void __launch_bounds__(256) out_grad_kernel(const float *yp, const fl
 {
     __shared__ float dy[OUT_ROWS];
     __shared__ float red[8][2][HID];
+    let_next_start();
+    wait_for_last();
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     float w[8], sw[8], sb[8], s3 = 0.0f, sl = 0.0f;
 #pragma unroll
@@ -372,6 +374,8 @@ __global__ void __launch_bounds__(256) out_grad_kernel(const float *yp, const fl
 __global__ void adam_kernel(float *p, const float *gr, float *m1, float *m2, uint64_t n, float lr, float b1t,
                             float b2t, bf16 *w1b, bf16 *w2b, bf16 *w1p, bf16 *w2p)
 {
+    let_next_start();
+    wait_for_last();
     for (uint64_t i = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; i < n; i += (uint64_t)gridDim.x * blockDim.x) {
         const float g = gr[i];
         const float a = 0.9f * m1[i] + 0.1f * g;
@@ -483,10 +487,10 @@ int backward(asse_mlp *m, const bf16 *x, const float *t, uint64_t n, float *loss
                        TcEpi{TE_BIAS_RELU_DOT, P + OFF_B2, P + OFF_W3, nullptr, m->H2, nullptr, m->y, HID}};
     MCK(m, launch_tc_gemm(&h2, 1, nothing, m->error, m->stream, &m->launches));
     const uint64_t ob = (n + OUT_ROWS - 1) / OUT_ROWS;
-    out_grad_kernel<<<(unsigned)(ob < 608 ? ob : 608), 256, 0, m->stream>>>(
-        m->y, P + OFF_B3, t, n, m->loss_kind, m->H2, P + OFF_W3, m->dZ2, G + OFF_W3, G + OFF_B2, G + OFF_B3, m->loss);
+    MCK(m, launch_dependent(out_grad_kernel, dim3((unsigned)(ob < 608 ? ob : 608)), 256, 0, m->stream, m->y, P + OFF_B3,
+                            t, n, m->loss_kind, m->H2, P + OFF_W3, m->dZ2, G + OFF_W3, G + OFF_B2, G + OFF_B3,
+                            m->loss));
     m->launches++;
-    MCK(m, cudaGetLastError());
     // the weight-gradient products reduce over the batch: split it so that
     // enough CTAs share the work
     const int splits = (int)((n + 255) / 256);
@@ -854,10 +858,9 @@ int asse_mlp_train_step(asse_mlp *m, const uint16_t *x_dev, const float *t_dev, 
         return rc;
     m->steps++;
     const float b1t = 1.0f - powf(0.9f, (float)m->steps), b2t = 1.0f - powf(0.999f, (float)m->steps);
-    adam_kernel<<<(unsigned)((NPARAMS + 255) / 256), 256, 0, m->stream>>>(
-        m->params, m->grads, m->m1, m->m2, NPARAMS, lr, b1t, b2t, m->w1b, m->w2b, m->w1p, m->w2p);
+    MCK(m, launch_dependent(adam_kernel, dim3((unsigned)((NPARAMS + 255) / 256)), 256, 0, m->stream, m->params, m->grads,
+                            m->m1, m->m2, NPARAMS, lr, b1t, b2t, m->w1b, m->w2b, m->w1p, m->w2p));
     m->launches++;
-    MCK(m, cudaGetLastError());
     return ASSE_OK;
 }
 

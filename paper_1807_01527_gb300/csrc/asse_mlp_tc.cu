@@ -565,11 +565,7 @@ __global__ void __launch_bounds__(TG_THREADS, 2) tc_gemm_kernel(const __grid_con
     const int m0 = blk % J.nx * 128, ny = blk / J.nx % J.ny, n0 = ny * BN, z = blk / (J.nx * J.ny);
     const int kb = z * J.kchunk, ke = min(J.p.K, kb + J.kchunk);
     const int nchunks = ke > kb ? (ke - kb + TG_KC - 1) / TG_KC : 0;
-    if (plans.extra.zero)
-        for (uint32_t i = blockIdx.x * TG_THREADS + tid; i < plans.extra.n_zero; i += gridDim.x * TG_THREADS)
-            plans.extra.zero[i] = 0.0f;
-    if (plans.extra.to && blockIdx.x == 0 && tid == 0)
-        *plans.extra.to = *plans.extra.from;
+    let_next_start();
     if (tid == 0) {
         for (int i = 0; i <= TG_STAGES; i++)
             mbar_init(&bar[i], 1);
@@ -583,6 +579,12 @@ __global__ void __launch_bounds__(TG_THREADS, 2) tc_gemm_kernel(const __grid_con
                      : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
+    wait_for_last();
+    if (plans.extra.zero)
+        for (uint32_t i = blockIdx.x * TG_THREADS + tid; i < plans.extra.n_zero; i += gridDim.x * TG_THREADS)
+            plans.extra.zero[i] = 0.0f;
+    if (plans.extra.to && blockIdx.x == 0 && tid == 0)
+        *plans.extra.to = *plans.extra.from;
     // this thread's 8 x 8 block of a transposed operand: of A in threads
     // 0..127, of B in the next BN (the first BN if A is not transposed)
     const bf16 *tp = nullptr;
@@ -818,9 +820,8 @@ cudaError_t launch_tc_gemm(const TcProduct *products, int count, const TcExtra &
     cudaError_t e = cudaFuncSetAttribute(tc_gemm_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess)
         return e;
-    tc_gemm_kernel<<<grid, TG_THREADS, smem, s>>>(plans, error);
     *launches += 1;
-    return cudaGetLastError();
+    return launch_dependent(tc_gemm_kernel, dim3(grid), TG_THREADS, smem, s, plans, error);
 }
 
 cudaError_t launch_mlp_pack(const float *params, bf16 *w1p, bf16 *w2p, cudaStream_t s, uint64_t *launches)

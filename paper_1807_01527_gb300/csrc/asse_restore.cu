@@ -308,6 +308,7 @@ __global__ void __launch_bounds__(RESTORE_THREADS) restore_kernel(Params P, cons
                                                                   const __grid_constant__ RestoreWindows out,
                                                                   uint64_t out_cap, SliceCtl *advance)
 {
+    wait_for_last();
     // the scan of this close has read the slice state; open the next slice
     if (advance != nullptr && blockIdx.x == 0 && blockIdx.y == 0)
         open_next_slice(P, advance);
@@ -428,8 +429,7 @@ cudaError_t launch_restores(const Params &P, const ScanWindows &W, uint32_t cap,
                             uint64_t out_cap, cudaStream_t s, uint64_t *launches, SliceCtl *advance)
 {
     *launches += 1;
-    restore_kernel<<<dim3(P.nf, W.n), RESTORE_THREADS, 0, s>>>(P, W, cap, out, out_cap, advance);
-    return cudaGetLastError();
+    return launch_dependent(restore_kernel, dim3(P.nf, W.n), RESTORE_THREADS, 0, s, P, W, cap, out, out_cap, advance);
 }
 
 cudaError_t launch_restore(const Params &P, const ScanOut &o, Tuple *scratch, uint32_t cap, asse_superpoint *csip,

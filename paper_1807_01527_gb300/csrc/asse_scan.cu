@@ -94,6 +94,7 @@ __global__ void __launch_bounds__(SCAN_THREADS, 4)
     }
     const typename L::Limit lim = L::limit(cyclic_vmax(P.ace != 0, P.k, L::W));
     __syncthreads();
+    wait_for_last();
 
     const uint32_t groups = 32 / lpa;        // ATVs side by side in a warp
     const uint32_t grp = lane / lpa, sub = lane - grp * lpa;
@@ -246,6 +247,7 @@ __global__ void __launch_bounds__(SCAN_THREADS, 4)
             }
         }
     }
+    let_next_start();
 }
 
 // ---------------------------------------------------------------- A3 alone
@@ -353,8 +355,7 @@ cudaError_t launch_scan_nw(const Params &P, uint32_t w, uint32_t *pool, const Sc
         const uint32_t per = 32 / lpa * SCAN_U * SCAN_WARPS;  // ATVs of a block's tiles
         const uint32_t want = (total + per - 1) / per;
         const uint32_t full = (uint32_t)sms * resident_blocks(kern, SCAN_THREADS, smem);
-        kern<<<want < full ? want : full, SCAN_THREADS, smem, s>>>(P, pool, W, ctl, total, lpa);
-        return cudaGetLastError();
+        return launch_dependent(kern, dim3(want < full ? want : full), SCAN_THREADS, smem, s, P, pool, W, ctl, total, lpa);
     });
 }
 
