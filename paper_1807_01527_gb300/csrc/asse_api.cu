@@ -254,9 +254,8 @@ int read_list(asse_pool *p, bool reported, asse_superpoint *out, uint64_t cap, u
         return fail(p, ASSE_EINVAL, "NULL argument");
     if (!p->restored)
         return fail(p, ASSE_ESTATE, "no restore since the last scan");
-    const bool early = reported && where != ASSE_DEVICE && p->report_host_valid;
     const HostReport host = host_report_w(p, p->sel);
-    if (!early) {
+    if (!p->report_host_valid) {
         CK(p, cudaMemcpyAsync(p->status_read, scan_out_w(p, p->sel).status, sizeof(Status), cudaMemcpyDeviceToHost,
                               p->stream));
         CK(p, cudaStreamSynchronize(p->stream));
@@ -265,7 +264,7 @@ int read_list(asse_pool *p, bool reported, asse_superpoint *out, uint64_t cap, u
         // next batch) keeps running
         CK(p, cudaEventSynchronize(p->close_done));
     }
-    const Status st = early ? *host.status : *p->status_read;
+    const Status st = p->report_host_valid ? *host.status : *p->status_read;
     if (st.overflow) {
         *n_out = st.needed;
         char buf[200];
@@ -276,7 +275,7 @@ int read_list(asse_pool *p, bool reported, asse_superpoint *out, uint64_t cap, u
     const uint64_t n = reported ? st.n_report : st.n_csip;
     *n_out = n;
     const uint64_t m = n < cap ? n : cap;
-    if (m > 0 && early && m <= p->report_host_cap) {
+    if (m > 0 && reported && where != ASSE_DEVICE && p->report_host_valid && m <= p->report_host_cap) {
         if (!out)
             return fail(p, ASSE_EINVAL, "out is NULL");
         memcpy(out, host.report, m * sizeof(asse_superpoint));
@@ -798,8 +797,16 @@ int asse_restore(asse_pool *p)
     if (int rc = wait_last_close(p))
         return rc;
     CK(p, launch_restore(p->P, scan_out(p), p->scratch, p->cap, p->csip, p->report, p->out_cap, p->stream,
-                         &p->launches));
+                         &p->launches, nullptr, host_report_w(p, 0)));
     p->restored = 1;
+    // as after a close, what the restore wrote for the host is there once it is
+    // done (a restore that the caller captures is read from the device)
+    cudaStreamCaptureStatus capturing = cudaStreamCaptureStatusNone;
+    CK(p, cudaStreamIsCapturing(p->stream, &capturing));
+    if (capturing == cudaStreamCaptureStatusNone) {
+        CK(p, cudaEventRecord(p->close_done, p->stream));
+        p->report_host_valid = 1;
+    }
     return ASSE_OK;
 }
 

@@ -321,7 +321,7 @@ __global__ void __launch_bounds__(RESTORE_THREADS) restore_kernel(Params P, cons
     __syncthreads();
     if (threadIdx.x == 0) {
         __threadfence();  // this block's counts before its own
-        if (atomicAdd(&o.status->done, 1u) + 1 == gridDim.x) {
+        if ((atomicAdd(&o.status->done, 1u) + 1) % gridDim.x == 0) {  // (of a repeated restore too)
             __threadfence();
             volatile Status *st = o.status;
             host.status->n_csip = st->n_csip;
