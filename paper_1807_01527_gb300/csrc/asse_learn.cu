@@ -503,7 +503,8 @@ int backward(asse_mlp *m, const bf16 *x, const float *t, uint64_t n, float *loss
          TcEpi{TE_RELU_GRAD, nullptr, nullptr, m->H1, m->dZ1, G + OFF_B1, nullptr, HID}}};
     MCK(m, launch_tc_gemm(hidden, 2, nothing, m->error, m->stream, &m->launches));
     // dW1[o][j] = sum_m dZ1[m][o] X[m][j]; this launch also hands the loss out
-    const TcProduct w1{TcOperand{m->dZ1, 1, HID}, TcOperand{x, 1, FEAT}, HID, FEAT, (int)n, splits,
+    // (two tiles only: split twice as far)
+    const TcProduct w1{TcOperand{m->dZ1, 1, HID}, TcOperand{x, 1, FEAT}, HID, FEAT, (int)n, (int)((n + 127) / 128),
                        TcEpi{TE_ATOMIC, nullptr, nullptr, nullptr, nullptr, G + OFF_W1, nullptr, FEAT}};
     MCK(m, launch_tc_gemm(&w1, 1, TcExtra{nullptr, 0, loss_dev, m->loss}, m->error, m->stream, &m->launches));
     return ASSE_OK;
