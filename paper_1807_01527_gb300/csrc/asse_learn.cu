@@ -263,8 +263,8 @@ __global__ void __launch_bounds__(SYNTH_WARPS * 32) synth_kernel(Params P, Synth
 
 // ---------------------------------------------------------------- elementwise
 
-// From the eight partial sums of every output (columns 32 q .. of the second
-// layer, q = 0..7; y = b3 + their sum) to the gradient of the second layer's
+// From the four partial sums of every output (columns 64 q .. of the second
+// layer, q = 0..3; y = b3 + their sum) to the gradient of the second layer's
 // outputs.  Squared error of the log: dy = 2 (y - t) / n, loss += (y - t)^2 / n.
 // Squared relative error of the estimate exp(y) against exp(t): with
 // e = exp(y - t), loss += (e - 1)^2 / n and dy = 2 (e - 1) e / n (y - t
@@ -300,7 +300,7 @@ __global__ void __launch_bounds__(256) out_grad_kernel(const float *yp, const fl
             if (m < n) {
                 float y = *b3;
 #pragma unroll
-                for (int q = 0; q < HID / 32; q++)
+                for (int q = 0; q < HID / 64; q++)
                     y += yp[q * n + m];
                 const float d = y - t[m];
                 if (kind == ASSE_LOSS_REL_MSE) {
@@ -419,7 +419,7 @@ struct asse_mlp {
     int *error = nullptr;                 // set by a kernel whose wait gave up
     uint64_t cap = 0;  // rows of the activation workspace
     bf16 *H1 = nullptr, *H2 = nullptr, *dZ2 = nullptr, *dZ1 = nullptr;
-    float *y = nullptr;     // partial sums of the outputs, HID / 32 per row
+    float *y = nullptr;     // partial sums of the outputs, HID / 64 per row
     float *loss = nullptr;  // after the gradients, in their allocation
     uint64_t steps = 0;
     int loss_kind = ASSE_LOSS_LOG_MSE;
@@ -464,7 +464,7 @@ int ensure_workspace(asse_mlp *m, uint64_t rows)
     MCK(m, cudaMalloc(&m->H2, act));
     MCK(m, cudaMalloc(&m->dZ2, act));
     MCK(m, cudaMalloc(&m->dZ1, act));
-    MCK(m, cudaMalloc(&m->y, rows * (HID / 32) * sizeof(float)));
+    MCK(m, cudaMalloc(&m->y, rows * (HID / 64) * sizeof(float)));
     m->cap = rows;
     return ASSE_OK;
 }

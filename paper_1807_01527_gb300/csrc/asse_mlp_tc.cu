@@ -682,7 +682,11 @@ __global__ void __launch_bounds__(TG_THREADS, 2) tc_gemm_kernel(const __grid_con
     if (done && nchunks > 0) {
         const int m = m0 + (warp & 3) * 32 + lane;
         const long row = (long)m * epi.ld;
-        for (int cb = warp / 4 * 32; cb < BN; cb += 64) {
+        // the last layer's dot product runs over a tile's 64 columns in order, so
+        // one warp takes both halves of its rows there
+        const bool whole = epi.kind == TE_BIAS_RELU_DOT;
+        float dot = 0.0f;
+        for (int cb = whole ? (warp < 4 ? 0 : BN) : warp / 4 * 32; cb < BN; cb += whole ? 32 : 64) {
             float v[32];
             __syncwarp();
             tmem_ld32(tmem + ((uint32_t)((warp & 3) * 32) << 16) + cb, v);
@@ -696,7 +700,6 @@ __global__ void __launch_bounds__(TG_THREADS, 2) tc_gemm_kernel(const __grid_con
                                       make_float4(v[j], v[j + 1], v[j + 2], v[j + 3]));
                 continue;
             }
-            float dot = 0.0f;
 #pragma unroll
             for (int j = 0; j < 32; j += 8) {
                 if (j >= cols || m >= M) {
@@ -732,8 +735,8 @@ __global__ void __launch_bounds__(TG_THREADS, 2) tc_gemm_kernel(const __grid_con
                                    fmaf(v[j + 2 * i], epi.w3[n + j + 2 * i], dot));
                 }
             }
-            if (epi.kind == TE_BIAS_RELU_DOT && m < M)
-                epi.y[(long)(n / 32) * M + m] = dot;
+            if (whole && cb + 32 >= BN && m < M)
+                epi.y[(long)ny * M + m] = dot;
             if (epi.kind == TE_RELU_GRAD) {
                 const float s = warp_column_sums(v, lane);
                 if (lane < cols)

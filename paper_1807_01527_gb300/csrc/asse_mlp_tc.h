@@ -41,7 +41,8 @@ __host__ __device__ inline uint32_t mlp_w2p_at(uint32_t n, uint32_t k)
 // split over `splits` CTAs (more than one only with TE_ATOMIC), and a fused
 // epilogue:
 //   TE_BIAS_RELU      out = bf16(relu(C + bias[n]))
-//   TE_BIAS_RELU_DOT  the same, and y[n / 32][m] = the 32 columns' sum of out * w3[n]
+//   TE_BIAS_RELU_DOT  the same, and y[t][m] = the sum of out * w3[n] over column tile t (64 columns
+//                     where N is a multiple of 64)
 //   TE_RELU_GRAD      out = bf16(C) where act > 0, else 0, and outf[n] += its column sums
 //   TE_ATOMIC         outf[m][n] += C (FP32 atomics)
 // with row stride ld (a multiple of 8; out, act and outf 16-byte aligned).  A
