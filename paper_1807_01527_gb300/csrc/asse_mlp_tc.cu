@@ -419,7 +419,7 @@ __global__ void __launch_bounds__(THREADS, 1)
 // The epilogue reads the accumulator with tcgen05.ld (warp w: rows 32 (w mod 4),
 // every other 32 columns) and applies the step's fused operation with 16-byte
 // accesses.  Two independent products share a launch (TcJobs).
-// Four Adam steps of 4,096 rows and the parameters read back: 1,073 -> 266 us
+// Four Adam steps of 4,096 rows and the parameters read back: 1,073 -> 244 us
 // (with the epilogues and the launches around, asse_learn.cu: 16 -> 6 a step);
 // the products took 35 us each with 2-byte gathers and stores.
 constexpr int TG_THREADS = 256;

@@ -5,7 +5,7 @@
 // admission: one for ingest (the kernel reads the batch size from device
 // memory, so one graph serves every batch size) and ASSE_SERVE_RING for the
 // close (reset, scan with the fused refresh, restore and estimate, advance of
-// the device-side slice state, copies of the status and report to pinned host
+// the device-side slice state, the status and report stored to pinned host
 // memory), one per report slot so up to ASSE_SERVE_RING closes of a stream
 // can be in flight.  Streams share the device and overlap freely; admission
 // charges each stream's device bytes against the server's budget.
@@ -45,7 +45,7 @@ struct SStream {
     uint32_t *staging = nullptr;
     unsigned long long *n_dev = nullptr;
     cudaGraphExec_t ingest = nullptr;
-    // one pinned host block for the status and report copies of every slot:
+    // one pinned host block for the status and report of every slot:
     // pinning host memory is slow and freeing it may wait for the device, so
     // a stream does each once, when it opens and when it closes
     unsigned char *pinned = nullptr;
