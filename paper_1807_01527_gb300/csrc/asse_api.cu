@@ -19,7 +19,7 @@ namespace {
 
 thread_local std::string g_create_error;
 
-constexpr uint64_t HOST_CHUNK = 1ull << 20;  // pairs of host input copied and ingested at a time
+constexpr uint64_t HOST_TAIL = 1ull << 20;  // pairs of host input ingested by themselves at the end of a batch
 
 struct SnapHeader {
     char magic[8];
@@ -66,6 +66,7 @@ struct asse_pool {
     SliceCtl *ctl = nullptr;  // device copy of the slice-dependent launch arguments
     uint32_t *stage[2] = {nullptr, nullptr};
     uint64_t stage_pairs = 0;
+    uint32_t stage_next = 0;  // the staging buffer of the next chunk
     uint32_t *q_aips = nullptr;
     asse_superpoint *q_out = nullptr;
     uint64_t q_cap = 0;
@@ -741,27 +742,34 @@ int asse_ingest(asse_pool *p, const uint32_t *pairs, uint64_t n, int where)
     // read pinned memory in place over the host link, but that keeps the SMs
     // busy for the whole transfer: 19.3 against 23.1 G pairs/s end to end on
     // the link workload with the next batch queued before each report.)
-    // Chunks of at most 8 MB: what follows the last copy is the ingest of the
-    // last chunk, 39 us for 4 Mi pairs (8 Mi pairs from pinned memory: 448 -> 434
-    // us a pass with chunks of 1 Mi), while a copy of 8 MB (41 us)
-    // still covers the ingest of the one before.
-    int last = -1;
-    const uint64_t chunk = p->stage_pairs < HOST_CHUNK ? p->stage_pairs : HOST_CHUNK;
-    for (uint64_t off = 0, i = 0; off < n; off += chunk, i++) {
-        const int b = (int)(i & 1);
-        const uint64_t m = (n - off) < chunk ? (n - off) : chunk;
+    // Chunks of a whole buffer, through the two in turn, from one call to the
+    // next: each boundary costs the copy engine about 2 us (chunks of 1 Mi
+    // pairs, the next batch queued before each report: 23.7 against 25.3 G
+    // pairs/s on the long workload, 23.1 against 23.9 on the link).  What follows
+    // the last copy, though, is the ingest of what it brought, so a last chunk of
+    // twice HOST_TAIL and more comes in two parts, the second of HOST_TAIL pairs
+    // (8 Mi pairs ingested, closed and reported before the next: 422 -> 399 us).
+    cudaEvent_t last = nullptr;
+    uint32_t part = 0;
+    for (uint64_t off = 0; off < n;) {
+        const uint32_t b = p->stage_next;
+        const uint64_t left = n - off, m = left < p->stage_pairs ? left : p->stage_pairs;
+        const uint64_t first = m == left && m >= 2 * HOST_TAIL ? (m - HOST_TAIL) / 2 * 2 : m;  // even: 16-byte aligned
         CK(p, cudaStreamWaitEvent(p->copy_stream, p->consumed[b], 0));
-        CK(p, cudaMemcpyAsync(p->stage[b], pairs + 2 * off, m * 8, cudaMemcpyHostToDevice, p->copy_stream));
-        CK(p, cudaEventRecord(p->copied[b], p->copy_stream));
-        CK(p, cudaStreamWaitEvent(p->stream, p->copied[b], 0));
-        CK(p, launch_ingest(p->P, p->w, p->pool, p->stage[b], m, nullptr, p->ctl, p->sms, p->stream,
-                            &p->launches));
+        for (uint64_t at = 0, k = first; at < m; at += k, k = m - at, part ^= 1) {
+            uint32_t *dst = p->stage[b] + 2 * at;
+            last = p->copied[part];
+            CK(p, cudaMemcpyAsync(dst, pairs + 2 * (off + at), k * 8, cudaMemcpyHostToDevice, p->copy_stream));
+            CK(p, cudaEventRecord(last, p->copy_stream));
+            CK(p, cudaStreamWaitEvent(p->stream, last, 0));
+            CK(p, launch_ingest(p->P, p->w, p->pool, dst, k, nullptr, p->ctl, p->sms, p->stream, &p->launches));
+        }
         CK(p, cudaEventRecord(p->consumed[b], p->stream));
-        last = b;
+        p->stage_next = b ^ 1;
+        off += m;
     }
     // the caller may reuse its host buffer once every chunk has been copied
-    if (last >= 0)
-        CK(p, cudaEventSynchronize(p->copied[last]));
+    CK(p, cudaEventSynchronize(last));
     return ASSE_OK;
 }
 
