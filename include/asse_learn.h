@@ -108,7 +108,8 @@ ASSE_API int asse_candidate_features(asse_pool *pool, const uint32_t *aips_dev, 
  * Eq. 4 estimate, flags and decision.  The reported candidates are written
  * to out (host or device, `where`) in unspecified order, min(count, cap) of
  * them, and *n_out receives the count.  Every step runs on the device; the
- * call synchronises the pool's stream (it reads the candidate count first).
+ * call synchronises the pool's stream (it reads the candidate count first, and
+ * waits for the copy to out).
  * Valid between asse_scan + asse_restore and asse_advance, as
  * asse_features (after asse_close_slice the refresh has changed the
  * state: ESTATE).  The model must use the pool's stream.  The library keeps

@@ -256,14 +256,13 @@ int read_list(asse_pool *p, bool reported, asse_superpoint *out, uint64_t cap, u
     if (!p->restored)
         return fail(p, ASSE_ESTATE, "no restore since the last scan");
     const HostReport host = host_report_w(p, p->sel);
+    // the close is done, on whichever stream; later work already queued (the
+    // next batch) keeps running
+    CK(p, cudaEventSynchronize(p->close_done));
     if (!p->report_host_valid) {
         CK(p, cudaMemcpyAsync(p->status_read, scan_out_w(p, p->sel).status, sizeof(Status), cudaMemcpyDeviceToHost,
                               p->stream));
         CK(p, cudaStreamSynchronize(p->stream));
-    } else {
-        // the close is done; later work already queued on the stream (the
-        // next batch) keeps running
-        CK(p, cudaEventSynchronize(p->close_done));
     }
     const Status st = p->report_host_valid ? *host.status : *p->status_read;
     if (st.overflow) {
@@ -285,8 +284,7 @@ int read_list(asse_pool *p, bool reported, asse_superpoint *out, uint64_t cap, u
             return fail(p, ASSE_EINVAL, "out is NULL");
         CK(p, cudaMemcpyAsync(out, list_w(p, p->sel, reported), m * sizeof(asse_superpoint),
                               where == ASSE_DEVICE ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost, p->stream));
-        if (where != ASSE_DEVICE)
-            CK(p, cudaStreamSynchronize(p->stream));
+        CK(p, cudaStreamSynchronize(p->stream));  // also of a device buffer, which any stream may read next
     }
     if (n > cap)
         return fail(p, ASSE_ECAPACITY, "output capacity smaller than the list");

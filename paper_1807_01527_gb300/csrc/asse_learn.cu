@@ -653,7 +653,7 @@ int asse_report_learned(asse_pool *pool, asse_mlp *m, float max_log_n, asse_supe
             return pool_fail(pool, ASSE_EINVAL, "out is NULL");
         e = cudaMemcpyAsync(out, rep, k * sizeof(asse_superpoint),
                             where == ASSE_DEVICE ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost, v.stream);
-        if (e == cudaSuccess && where != ASSE_DEVICE)
+        if (e == cudaSuccess)
             e = cudaStreamSynchronize(v.stream);
         if (e != cudaSuccess)
             return pool_fail(pool, ASSE_ECUDA, std::string("learned report copy: ") + cudaGetErrorString(e));
