@@ -58,6 +58,7 @@ struct asse_pool {
     asse_superpoint *report_host = nullptr;
     uint64_t report_host_cap = 0;
     int report_host_valid = 0;
+    int captured = 0;  // a graph of the caller's holds a restore of this pool
     cudaEvent_t close_done = nullptr;  // recorded after the last close
     Status *status_read = nullptr;     // pinned, for reading any other status
     // asse_set_timing: events around the scan and the restore of each close
@@ -231,6 +232,29 @@ HostReport host_report_w(asse_pool *p, uint32_t m)
 {
     return m == 0 ? HostReport{p->status_host, p->report_host, p->report_host_cap}
                   : HostReport{p->win[m - 1].status_host, p->win[m - 1].report_host, p->report_host_cap};
+}
+
+// Whether the pool's stream is being captured.  The graph may be replayed at any
+// time, also while the host reads a report, so a restore in it writes device
+// memory only (HostReport()), records no event, and from then on the readers take
+// status and lists from the device.
+int check_capture(asse_pool *p, bool *capturing)
+{
+    cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+    CK(p, cudaStreamIsCapturing(p->stream, &st));
+    *capturing = st != cudaStreamCaptureStatusNone;
+    return ASSE_OK;
+}
+
+// After the restore of a close or of asse_restore is queued.
+int note_restore(asse_pool *p, bool capturing)
+{
+    if (capturing)
+        p->captured = 1;
+    else
+        CK(p, cudaEventRecord(p->close_done, p->stream));
+    p->report_host_valid = !p->captured;
+    return ASSE_OK;
 }
 
 int reset_close_state(asse_pool *p)
@@ -800,20 +824,15 @@ int asse_restore(asse_pool *p)
     if (!p->scanned)
         return fail(p, ASSE_ESTATE, "restore needs a scan of the open slice");
     p->report_host_valid = 0;
+    bool capturing = false;
+    if (int rc = check_capture(p, &capturing))
+        return rc;
     if (int rc = wait_last_close(p))
         return rc;
     CK(p, launch_restore(p->P, scan_out(p), p->scratch, p->cap, p->csip, p->report, p->out_cap, p->stream,
-                         &p->launches, nullptr, host_report_w(p, 0)));
+                         &p->launches, nullptr, capturing ? HostReport() : host_report_w(p, 0)));
     p->restored = 1;
-    // as after a close, what the restore wrote for the host is there once it is
-    // done (a restore that the caller captures is read from the device)
-    cudaStreamCaptureStatus capturing = cudaStreamCaptureStatusNone;
-    CK(p, cudaStreamIsCapturing(p->stream, &capturing));
-    if (capturing == cudaStreamCaptureStatusNone) {
-        CK(p, cudaEventRecord(p->close_done, p->stream));
-        p->report_host_valid = 1;
-    }
-    return ASSE_OK;
+    return note_restore(p, capturing);
 }
 
 int asse_advance(asse_pool *p)
@@ -833,15 +852,16 @@ int asse_close_slice(asse_pool *p, uint32_t kp)
         return fail(nullptr, ASSE_EINVAL, "pool is NULL");
     if (int rc = check_kp(p, kp))
         return rc;
+    bool capturing = false;
+    if (int rc = check_capture(p, &capturing))
+        return rc;
     if (int rc = wait_last_close(p))
         return rc;
-    if (int rc = pool_enqueue_close(p, kp, host_report_w(p, 0), p->timing != 0))
+    if (int rc = pool_enqueue_close(p, kp, capturing ? HostReport() : host_report_w(p, 0), p->timing != 0))
         return rc;
     pool_after_close(p, kp);
     p->timed = p->timing;
-    CK(p, cudaEventRecord(p->close_done, p->stream));
-    p->report_host_valid = 1;
-    return ASSE_OK;
+    return note_restore(p, capturing);
 }
 
 int asse_close_slice_multi(asse_pool *p, const uint32_t *kps, uint32_t n_windows)
@@ -895,6 +915,9 @@ int asse_close_slice_multi(asse_pool *p, const uint32_t *kps, uint32_t n_windows
         w.report = reinterpret_cast<asse_superpoint *>(w.block + report);
         w.scratch = reinterpret_cast<Tuple *>(w.block + scratch);
     }
+    bool capturing = false;
+    if (int rc = check_capture(p, &capturing))
+        return rc;
     if (int rc = wait_last_close(p))
         return rc;
     ScanWindows W{};
@@ -904,7 +927,7 @@ int asse_close_slice_multi(asse_pool *p, const uint32_t *kps, uint32_t n_windows
         W.kp[m] = kps[m];
         W.o[m] = scan_out_w(p, m);
         out.w[m] = RestoreOut{m == 0 ? p->scratch : p->win[m - 1].scratch, list_w(p, m, false), list_w(p, m, true),
-                              host_report_w(p, m)};
+                              capturing ? HostReport() : host_report_w(p, m)};
     }
     CK(p, launch_reset(W, p->cfg.r * p->P.nf, p->stream, &p->launches));
     if (p->P.hist) {
@@ -922,9 +945,7 @@ int asse_close_slice_multi(asse_pool *p, const uint32_t *kps, uint32_t n_windows
     }
     pool_after_close(p, kps[0]);
     p->n_windows = n_windows;
-    CK(p, cudaEventRecord(p->close_done, p->stream));
-    p->report_host_valid = 1;
-    return ASSE_OK;
+    return note_restore(p, capturing);
 }
 
 int asse_set_timing(asse_pool *p, int on)
