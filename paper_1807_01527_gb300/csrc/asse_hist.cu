@@ -78,6 +78,7 @@ __global__ void __launch_bounds__(HIST_THREADS) hist_scan_kernel(Params P, uint3
     RangeDesc *desc = reinterpret_cast<RangeDesc *>(hsm);                  // [Wd] count ranges
     RangeDesc *rdesc = desc + P.Wd;                                        // [Wd] refresh ranges (FUSE)
     uint32_t *maskbuf = reinterpret_cast<uint32_t *>(rdesc + (FUSE ? P.Wd : 0));  // [warps][mw]
+    wait_for_last();
     const uint32_t c0 = ctl->c0;
     const Refresh R = ctl->R;
     const uint32_t lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -87,7 +88,6 @@ __global__ void __launch_bounds__(HIST_THREADS) hist_scan_kernel(Params P, uint3
             rdesc[q] = refresh_desc<WB>(P, q, R.c0n);
     }
     __syncthreads();
-    wait_for_last();
     uint32_t *my_mask = maskbuf + warp * P.mw;
     // the refreshed words as up to four slots when the (at most two) ranges
     // hold at most four words together

@@ -473,8 +473,8 @@ __global__ void advance_ctl_kernel(Params P, SliceCtl *ctl)
 
 __global__ void reset_kernel(const __grid_constant__ ScanWindows W, uint32_t nseg)
 {
-    // the scan may start its set-up, which reads the slice state, only once
-    // what wrote that is over
+    // in this order, as the other would let the scan's blocks sit on the SMs
+    // while an ingest is still running
     wait_for_last();
     let_next_start();
     const ScanOut o = W.o[blockIdx.y];

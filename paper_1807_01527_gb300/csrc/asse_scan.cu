@@ -71,8 +71,6 @@ __global__ void __launch_bounds__(SCAN_THREADS, 4)
     scan_kernel(Params P, uint32_t *pool, const ScanWindows W, const SliceCtl *ctl, uint32_t total_atv, uint32_t lpa)
 {
     static_assert(!BG || WB == 8, "the in-field guard needs byte-wide fields");
-    const uint32_t c0 = ctl->c0;
-    const Refresh &R = ctl->R;
     extern __shared__ __align__(128) uint8_t smem[];
     const uint32_t nw = NW == 1 ? 1u : W.n;
     const uint32_t nchunk = P.Wd / 4;
@@ -86,6 +84,9 @@ __global__ void __launch_bounds__(SCAN_THREADS, 4)
     uint32_t *maskbuf = reinterpret_cast<uint32_t *>(rd + P.Wd);      // [warps][mw]
 
     const uint32_t tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    wait_for_last();
+    const uint32_t c0 = ctl->c0;
+    const Refresh &R = ctl->R;
     for (uint32_t e = tid; e < nw * P.Wd; e += SCAN_THREADS) {
         const uint32_t m = e / P.Wd, q = e - m * P.Wd;
         cd[didx(m, q)] = cyclic_count_entry<WB, BG>(P, q, c0, W.kp[m]);
@@ -94,7 +95,6 @@ __global__ void __launch_bounds__(SCAN_THREADS, 4)
     }
     const typename L::Limit lim = L::limit(cyclic_vmax(P.ace != 0, P.k, L::W));
     __syncthreads();
-    wait_for_last();
 
     const uint32_t groups = 32 / lpa;        // ATVs side by side in a warp
     const uint32_t grp = lane / lpa, sub = lane - grp * lpa;
