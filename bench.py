@@ -275,6 +275,7 @@ def stepwise_breakdown(pool, dev, w, n):
         pool.advance()
         e[4].record(stream)
         pool.report()
+        e[4].synchronize()      # the report has waited for the restore alone
         for name, a, b in (("ingest", 0, 1), ("scan", 1, 2), ("restore", 2, 3), ("refresh", 3, 4)):
             acc[name].append(e[a].elapsed_time(e[b]))
         f0 = torch.cuda.Event(enable_timing=True)
@@ -284,6 +285,7 @@ def stepwise_breakdown(pool, dev, w, n):
         pool.close_slice(w.k)
         f1.record(stream)
         pool.report()
+        f1.synchronize()
         acc["fused_close"].append(f0.elapsed_time(f1))
     return {k: statistics.mean(v) for k, v in acc.items()}
 
