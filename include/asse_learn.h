@@ -75,7 +75,8 @@ ASSE_API int asse_estimate_learned(asse_pool *pool, asse_mlp *mlp, float max_log
 /* States first .. first+n-1 of a synthetic set: features x_dev [n][FEAT]
  * bf16, labels log_n_dev [n] = ln(n) and the Eq. 2 estimate of each state's
  * count lc_dev [n] (a saturated count g is taken as g - 1/2).  All device
- * buffers; stream-ordered on stream.  Errors: EINVAL, ECUDA. */
+ * buffers; stream-ordered on stream.  Errors: EINVAL (also g > 3712 with
+ * k >= 32), ECUDA. */
 ASSE_API int asse_synth_states(const asse_synth_cfg *cfg, uint64_t first, uint64_t n, uint16_t *x_dev,
                                float *log_n_dev, float *lc_dev, void *stream);
 

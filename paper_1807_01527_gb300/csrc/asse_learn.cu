@@ -153,7 +153,7 @@ __host__ __device__ inline size_t synth_smem(uint32_t k, uint32_t g, uint32_t ba
 // 16,384 states of k = 10, g = 512, n up to 2^20: 2,290 us with a block a
 // state and every draw made, 200 us now.
 __global__ void __launch_bounds__(SYNTH_WARPS * 32) synth_kernel(Params P, SynthArgs S, uint64_t first, uint64_t n,
-                                                                 uint32_t batch, uint32_t visible, int table, bf16 *x,
+                                                                 uint32_t batch, int table, bf16 *x,
                                                                  float *log_n, float *lc)
 {
     extern __shared__ double synth_sm[];
@@ -240,7 +240,7 @@ __global__ void __launch_bounds__(SYNTH_WARPS * 32) synth_kernel(Params P, Synth
                     if ((splitmix(bkey ^ ix) >> 11) < lim)
                         l = t;
                 }
-                if (l >= 0 && at_pos(P, h) < visible) {
+                if (l >= 0) {
                     hist[(k - 1 - (uint32_t)l) * 32 + lane] += 1;
                     cnt++;
                 }
@@ -673,24 +673,16 @@ int asse_synth_states(const asse_synth_cfg *cfg, uint64_t first, uint64_t n, uin
         return ASSE_EINVAL;
     if (n == 0)
         return ASSE_OK;
+    // an ATV of at most 928 words: 3,712 byte-wide fields
+    if (cfg->g > 928 * (32 / packed_width(ASSE_COUNTER_AT, cfg->k)))
+        return ASSE_EINVAL;
     Params P{};
     P.k = cfg->k;
-    P.k2 = 2 * cfg->k;
     P.g = cfg->g;
     P.r = cfg->r;
-    P.blk = cfg->g / (2 * cfg->k);
-    P.blk_magic = ((1ull << 32) + P.blk - 1) / P.blk;
-    P.paired = 1;  // the storage order of a timestamp pool's ACT blocks
     P.bh_a = cfg->bh_a;
     P.bh_b = cfg->bh_b;
-    const uint32_t w = packed_width(ASSE_COUNTER_AT, cfg->k);
-    const uint32_t Fw = 32 / w;
-    P.Wd = ((cfg->g + Fw - 1) / Fw + 7) / 8 * 8;
     SynthArgs S{cfg->seed, cfg->n_max_log2, cfg->bg_max};
-    // ATVs of more than 933 words (g above 3,712 in byte-wide fields) are refused
-    if (P.Wd > 933)
-        return ASSE_ECUDA;
-    const uint32_t visible = 512 * Fw;  // a feature row counts the first 512 words of an ATV, all a pool's can have
     int dev = 0, sms = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
@@ -703,7 +695,7 @@ int asse_synth_states(const asse_synth_cfg *cfg, uint64_t first, uint64_t n, uin
     cudaError_t e = cudaFuncSetAttribute(synth_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e == cudaSuccess) {
         synth_kernel<<<(unsigned)(blocks < (1u << 30) ? blocks : (1u << 30)), SYNTH_WARPS * 32, smem,
-                       (cudaStream_t)stream>>>(P, S, first, n, batch, visible, table ? 1 : 0,
+                       (cudaStream_t)stream>>>(P, S, first, n, batch, table ? 1 : 0,
                                                reinterpret_cast<bf16 *>(x_dev), log_n_dev, lc_dev);
         e = cudaGetLastError();
     }
