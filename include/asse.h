@@ -122,7 +122,9 @@ extern "C" {
  *          keeps one when the pool is larger than the device's L2 cache (the
  *          repeats then cost DRAM sectors), and, where the memory for it can
  *          be had, for every other pool but those with slice counts and those
- *          of a server.  Results are the same either way.
+ *          of a server; these others use it only while the open slice has taken
+ *          no more than 2 pairs per AT of a row (4 where the fields are 8 bits
+ *          wide).  Results are the same either way.
  *  cluster CTAs of a thread-block cluster that share one table of the keys
  *          their ingest has seen (each CTA's shared-memory table holds the
  *          keys that hash to it, reached by the others through distributed

@@ -68,6 +68,8 @@ struct asse_pool {
     uint32_t *stage[2] = {nullptr, nullptr};
     uint64_t stage_pairs = 0;
     uint32_t stage_next = 0;  // the staging buffer of the next chunk
+    uint64_t slice_pairs = 0;   // ingested into the open slice
+    uint64_t claim_pairs = ~0ull;  // so many at most go through a key table the pool could do without
     uint32_t *q_aips = nullptr;
     asse_superpoint *q_out = nullptr;
     uint64_t q_cap = 0;
@@ -451,6 +453,7 @@ void pool_after_close(asse_pool *p, uint32_t kp)
     p->scan_kp = kp;
     p->scan_slice = p->t;
     p->t += 1;
+    p->slice_pairs = 0;
 }
 
 int pool_enqueue_ingest(asse_pool *p, const uint32_t *pairs_dev, const unsigned long long *n_dev)
@@ -472,6 +475,19 @@ uint32_t pool_restore_cap(const asse_pool *p) { return p->cap; }
 static bool key_table_pays(const asse_config *cfg)
 {
     return cfg->key_table == ASSE_KEYS_AUTO && cfg->counter != ASSE_COUNTER_AT_HIST;
+}
+
+// Pairs of a slice up to which such a table is used: two per AT of a row, four
+// where the fields are bytes, whose blind set is one store.  A slice of many more
+// distinct keys than fields finds most fields set, and its keys push one another
+// out of the table, so that claiming each and setting it blind costs more than
+// reading its words.  With / without the table, us, 8.4 M pairs of random hosts:
+// 4 pairs per AT 457 / 208 (five bits, 4,096 ATVs a row), 64 per AT 517 / 132 (four
+// bits, 1,024); of the workloads' Zipf hosts 102 / 88 and 113 / 68.  At one pair
+// per AT it is 463 / 411 and 95 / 98, at a half 69 / 57 and 22 / 29.
+static uint64_t claim_pairs(const Params &P, uint32_t w)
+{
+    return ((uint64_t)P.g << P.E_log2) * (w == 8 ? 4 : 2);
 }
 
 // log2 entries of the key table asse_create cannot do without on the current
@@ -658,6 +674,8 @@ int asse_create(const asse_config *cfg, void *stream, asse_pool **out)
             cudaGetLastError();
             P.keys = nullptr;
             P.klg = 0;
+        } else {
+            p->claim_pairs = claim_pairs(P, p->w);
         }
     }
     if (e == cudaSuccess)
@@ -749,14 +767,18 @@ int asse_ingest(asse_pool *p, const uint32_t *pairs, uint64_t n, int where)
     if (!pairs)
         return fail(p, ASSE_EINVAL, "pairs is NULL");
     p->ingested = 1;  // the pool no longer matches the last scan
+    if (where != ASSE_HOST && where != ASSE_DEVICE)
+        return fail(p, ASSE_EINVAL, "where must be ASSE_HOST or ASSE_DEVICE");
+    if (where == ASSE_DEVICE && ((uintptr_t)pairs & 15) != 0)
+        return fail(p, ASSE_EINVAL, "device pairs must be 16-byte aligned");
+    p->slice_pairs += n;
+    Params P = p->P;
+    if (p->slice_pairs > p->claim_pairs)
+        P.keys = nullptr;
     if (where == ASSE_DEVICE) {
-        if (((uintptr_t)pairs & 15) != 0)
-            return fail(p, ASSE_EINVAL, "device pairs must be 16-byte aligned");
-        CK(p, launch_ingest(p->P, p->w, p->pool, pairs, n, nullptr, p->ctl, p->sms, p->stream, &p->launches));
+        CK(p, launch_ingest(P, p->w, p->pool, pairs, n, nullptr, p->ctl, p->sms, p->stream, &p->launches));
         return ASSE_OK;
     }
-    if (where != ASSE_HOST)
-        return fail(p, ASSE_EINVAL, "where must be ASSE_HOST or ASSE_DEVICE");
     // Double-buffered staging (Sec. 4.4): the copy engines move chunk i+1 on
     // the copy stream while chunk i is ingested on the pool's stream, and the
     // call returns once the last chunk is copied, so the ingest and the close
@@ -784,7 +806,7 @@ int asse_ingest(asse_pool *p, const uint32_t *pairs, uint64_t n, int where)
             CK(p, cudaMemcpyAsync(dst, pairs + 2 * (off + at), k * 8, cudaMemcpyHostToDevice, p->copy_stream));
             CK(p, cudaEventRecord(last, p->copy_stream));
             CK(p, cudaStreamWaitEvent(p->stream, last, 0));
-            CK(p, launch_ingest(p->P, p->w, p->pool, dst, k, nullptr, p->ctl, p->sms, p->stream, &p->launches));
+            CK(p, launch_ingest(P, p->w, p->pool, dst, k, nullptr, p->ctl, p->sms, p->stream, &p->launches));
         }
         CK(p, cudaEventRecord(p->consumed[b], p->stream));
         p->stage_next = b ^ 1;
@@ -842,6 +864,7 @@ int asse_advance(asse_pool *p)
     CK(p, launch_refresh(p->P, p->w, p->pool, p->ctl, p->sms, p->stream, &p->launches));
     CK(p, launch_advance_ctl(p->P, p->ctl, p->stream, &p->launches));
     p->t += 1;
+    p->slice_pairs = 0;
     p->refreshed = 1;
     return ASSE_OK;
 }
@@ -1151,6 +1174,7 @@ int asse_load(asse_pool *p, const void *src, uint64_t n)
         CK(p, launch_hist_rebuild(p->P, p->w, p->pool, p->ctl, p->sms, p->stream, &p->launches));
     CK(p, cudaStreamSynchronize(p->stream));
     p->t = h.slice;
+    p->slice_pairs = 0;
     p->scanned = p->restored = p->refreshed = 0;
     return ASSE_OK;
 }
