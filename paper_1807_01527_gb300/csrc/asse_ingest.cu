@@ -206,8 +206,8 @@ __device__ __forceinline__ void set_field_hist(const Params &P, uint32_t *addr, 
 
 // How a launch sets the fields of a key, a template parameter of the kernel.
 enum SetKind {
-    SET_READ,       // no key table: read each word, change only a field that does not hold the value yet
-    SET_BLIND,      // the key was claimed in the key table: set its fields without reading them
+    SET_READ,       // read each word, change only a field that does not hold the value yet
+    SET_BLIND,      // the key was claimed in the key table: set its fields without reading them (P.blind)
     SET_READ_HIST   // slice counts: read, compare-and-swap (the counts need the old value)
 };
 
@@ -427,8 +427,8 @@ cudaError_t launch_ingest(const Params &P, uint32_t w, uint32_t *pool, const uin
                             : (P.r == 4 ? ingest_kernel<WB, 4, SET, false> : ingest_kernel<WB, 0, SET, false>);
         };
         auto kern = P.hist ? pick(std::integral_constant<int, SET_READ_HIST>())
-                    : P.keys ? pick(std::integral_constant<int, SET_BLIND>())
-                             : pick(std::integral_constant<int, SET_READ>());
+                    : P.keys && P.blind ? pick(std::integral_constant<int, SET_BLIND>())
+                                        : pick(std::integral_constant<int, SET_READ>());
         cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess)
             return e;

@@ -35,6 +35,7 @@ struct Params {
     // 32 bits of the slice (all ones = empty).  Null for a pool without one.
     unsigned long long *keys;
     uint32_t klg;
+    uint32_t blind;  // the fields of a claimed key are set without reading them
     // ASSE_COUNTER_AT_HIST: per ATV, the ATs last set in each slice phase
     // t mod 2k, phase-major ([2k][r * E] 16-bit counts); null otherwise.
     uint16_t *hist;

@@ -50,3 +50,38 @@ def test_batches_across_the_line(mods, counter, k, g, per_at):
         orc.advance()
         np.testing.assert_array_equal(state(pool), orc.at(), err_msg="after slice %d" % t)
     pool.close()
+
+
+@pytest.mark.parametrize("counter,k,g,elog,ats_per_pair", [("at", 60, 288, 17, 5), ("at", 10, 512, 17, 10),
+                                                           ("ace", 10, 512, 18, 10)])
+def test_large_pool_across_its_line(mods, counter, k, g, elog, ats_per_pair):
+    """A pool larger than the L2 cache, whose claimed keys are set blind up to a
+    line and read first past it, equals one without a key table; the keys of one
+    batch come again in the others."""
+    asse, oracle, torch = mods
+    c, u, s = synth.column_split(elog, 4)
+    p = dict(k=k, theta=g, g=g, r=4, c=c, u=u, s=s, **synth.method_keys(k + g))
+    pools = [asse.Pool(p, counter=counter, key_table=kt) for kt in ("auto", "off")]
+    l2 = torch.cuda.get_device_properties(0).L2_cache_size
+    assert 4 * pools[0].info()["pool_words"] > l2
+    line = (g << elog) // ats_per_pair
+    gen = torch.Generator(device="cuda").manual_seed(k)
+    for t in range(2):
+        x = torch.randint(-(1 << 31), 1 << 31, (line + 300_001, 2), generator=gen, device="cuda",
+                          dtype=torch.int64).to(torch.int32)
+        x[:, 0] %= 5003
+        x[:, 1] %= 2003
+        batches = [x[: line // 2], x[line // 2: line], x[line: line + 1], x[line + 1:], x[: 100_001]]
+        for b in batches:
+            b = b.clone()               # from a 16-byte boundary
+            for pool in pools:
+                pool.ingest(b)
+            torch.cuda.synchronize()
+        a, b = (pool.read_pool() for pool in pools)
+        np.testing.assert_array_equal(a, b, err_msg="slice %d" % t)
+        for pool in pools:
+            pool.close_slice()
+        np.testing.assert_array_equal(pools[0].counts(), pools[1].counts())
+        assert (pools[0].counts() > 0).any()
+    for pool in pools:
+        pool.close()
