@@ -113,8 +113,8 @@ extern "C" {
  *          restore; 0 selects 4096.  The candidate lists hold up to
  *          restore_cap * 2^u entries.
  *  max_batch    device staging capacity in pairs for ASSE_HOST ingest
- *          (copied in chunks of this size, through two such buffers); 0 selects
- *          4 Mi.
+ *          (copied in chunks of up to this size, through two such buffers); 0
+ *          selects 4 Mi.
  *  key_table    ASSE_KEYS_AUTO, ASSE_KEYS_ON or ASSE_KEYS_OFF: whether the
  *          ingest keeps a device table of the (aip, BH(bip)) keys already set
  *          in the open slice (4 entries of 8 bytes per ATV, 1 to 32 MiB), so
@@ -203,8 +203,8 @@ ASSE_API int asse_set_stream(asse_pool *pool, void *stream);
  *   ASSE_DEVICE: a device address, 16-byte aligned, that must stay valid
  *   until the stream reaches this work; nothing is copied.
  *   ASSE_HOST: host memory (pinned memory gives full copy-engine bandwidth),
- *   copied in chunks of max_batch pairs (of a last one of 2 Mi pairs and more
- *   the last 1 Mi by themselves) into device staging, the copy of chunk i+1
+ *   copied in chunks of up to max_batch pairs (the last up to 1 Mi of more than
+ *   1.25 Mi by themselves) into device staging, the copy of chunk i+1
  *   overlapping the ingest of chunk i.  The call returns once the last chunk
  *   is copied: the host buffer may then be reused, and the ingest of the last
  *   chunk (and a close queued after it) run on while the caller prepares its

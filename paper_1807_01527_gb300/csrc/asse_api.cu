@@ -19,7 +19,28 @@ namespace {
 
 thread_local std::string g_create_error;
 
-constexpr uint64_t HOST_TAIL = 1ull << 20;  // pairs of host input ingested by themselves at the end of a batch
+// Host input comes in chunks of up to a staging buffer, the last one, if it has more
+// than HOST_SPLIT pairs, in two parts: the second of at most HOST_TAIL pairs.  Both
+// start at multiples of HOST_ALIGN pairs.
+constexpr uint64_t HOST_TAIL = 1ull << 20, HOST_SPLIT = 5ull << 18, HOST_ALIGN = 1ull << 16;
+
+uint64_t host_aligned(uint64_t pairs) { return (pairs + HOST_ALIGN - 1) / HOST_ALIGN * HOST_ALIGN; }
+
+// Pairs of the next chunk, left pairs from the end: a buffer of stage pairs
+// (even), or half of what is left where that fits in the two.
+uint64_t host_chunk(uint64_t left, uint64_t stage)
+{
+    if (left <= stage)
+        return left;
+    const uint64_t half = host_aligned(left / 2);
+    return left < 2 * stage && half < stage ? half : stage;
+}
+
+// Pairs of the first part of a last chunk of m pairs.
+uint64_t host_first(uint64_t m)
+{
+    return m <= HOST_SPLIT ? m : m < 2 * HOST_TAIL ? HOST_TAIL : host_aligned(m - HOST_TAIL);
+}
 
 struct SnapHeader {
     char magic[8];
@@ -168,7 +189,8 @@ int validate(const asse_config *c, std::string &why)
         return bad("key_table must be ASSE_KEYS_AUTO, ASSE_KEYS_ON or ASSE_KEYS_OFF");
     if (c->cluster != ASSE_CLUSTER_AUTO && c->cluster != 1 && c->cluster != 2 && c->cluster != 4 && c->cluster != 8)
         return bad("cluster must be ASSE_CLUSTER_AUTO, 1, 2, 4 or 8");
-    // the scan holds one ATV in a warp tile of at most 512 words
+    // the scan and the estimates keep an entry per word of an ATV in shared
+    // memory (of up to four windows and the refresh: 40 KB for 512 words)
     const uint32_t w = packed_width(c->counter, c->k);
     if ((c->g + 32 / w - 1) / (32 / w) > 512)
         return bad("an ATV must fit in 512 words: need g <= 512 * floor(32 / w)");
@@ -807,15 +829,15 @@ int asse_ingest(asse_pool *p, const uint32_t *pairs, uint64_t n, int where)
     // next: each boundary costs the copy engine about 2 us (chunks of 1 Mi
     // pairs, the next batch queued before each report: 23.7 against 25.3 G
     // pairs/s on the long workload, 23.1 against 23.9 on the link).  What follows
-    // the last copy, though, is the ingest of what it brought, so a last chunk of
-    // twice HOST_TAIL and more comes in two parts, the second of HOST_TAIL pairs
-    // (8 Mi pairs ingested, closed and reported before the next: 422 -> 399 us).
+    // the last copy, though, is the ingest of what it brought, so the last chunk
+    // comes in two parts (host_first; 8 Mi pairs ingested, closed and reported
+    // before the next: 422 -> 399 us).
     cudaEvent_t last = nullptr;
     uint32_t part = 0;
     for (uint64_t off = 0; off < n;) {
         const uint32_t b = p->stage_next;
-        const uint64_t left = n - off, m = left < p->stage_pairs ? left : p->stage_pairs;
-        const uint64_t first = m == left && m >= 2 * HOST_TAIL ? (m - HOST_TAIL) / 2 * 2 : m;  // even: 16-byte aligned
+        const uint64_t m = host_chunk(n - off, p->stage_pairs);
+        const uint64_t first = m == n - off ? host_first(m) : m;
         CK(p, cudaStreamWaitEvent(p->copy_stream, p->consumed[b], 0));
         for (uint64_t at = 0, k = first; at < m; at += k, k = m - at, part ^= 1) {
             uint32_t *dst = p->stage[b] + 2 * at;

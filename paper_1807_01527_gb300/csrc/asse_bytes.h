@@ -1,10 +1,12 @@
-// Word-level tests on byte-wide counter fields whose values stay below 128:
+// Word-level operations on byte-wide counter fields whose values stay below 128:
 // the packed layout of seven-bit counters, which packed_width
 // (asse_internal.h) stores in eight bits, four fields to a 32-bit word.  Bit
 // 7 of every byte is 0 in the pool, so it serves as the guard bit in place:
 // one subtraction tests all four fields against a bound, with no borrow
 // from one byte into the next.  Host and device code (the host build checks
-// these functions exhaustively against per-byte definitions).
+// these functions exhaustively against per-byte definitions).  The kernels use
+// decay_bytes; their range tests are one cyclic range per field (asse_cyclic.h),
+// the two-range ones here the plain form of the same tests, for the host check.
 #pragma once
 
 #include <cstdint>

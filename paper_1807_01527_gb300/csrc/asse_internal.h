@@ -82,7 +82,7 @@ __device__ __forceinline__ void hist_add(uint16_t *hist, uint64_t i, int delta)
 // for aging counters (values 0..k), except that 7 becomes 8.  A word holds
 // floor(32/7) = floor(32/8) = 4 fields either way, so the byte-wide fields
 // cost no memory, and their top bit, never set by a 7-bit value, lets one
-// SWAR step test all four fields of a word (asse_swar.cuh).
+// SWAR step test all four fields of a word (asse_cyclic.h).
 inline uint32_t packed_width(uint32_t counter, uint32_t k)
 {
     uint32_t v = counter == ASSE_COUNTER_ACE ? k + 1 : 2 * k + 1, b = 0;

@@ -1,15 +1,17 @@
-// SWAR activity tests on packed AT words, shared by the scan (asse_scan.cu)
-// and the feature rows of the learned estimator (asse_features.cu).
+// SWAR tests on packed AT words: with two plain ranges per field, for the
+// slice-count scan (asse_hist.cu) and the candidate feature rows
+// (asse_candidates.cu, asse_features.cuh); with one cyclic range
+// (asse_cyclic.h), for the scan and the estimates (asse_scan.cu,
+// asse_restore.cu); and the aging counters' decrement.
 //
-// The active values of a block form the cyclic window act-k'+1 .. act (mod
+// Two ranges: the active values of a block form the cyclic window act-k'+1 .. act (mod
 // 2k), i.e. at most two plain ranges.  The even and the odd fields of a word
 // are tested separately, each field then having w free bits above it; with
 // a guard bit just above each field, (v | guard) - lo keeps the guard iff
 // v >= lo and (hi | guard) - v keeps it iff v <= hi, with no borrow between
 // fields.  Per-position constants carry each field's own range, so words
 // that straddle two ACT blocks and the fields past g (empty ranges) need no
-// special case.  Byte-wide fields holding seven-bit values have the guard
-// bit inside the field and are tested all four at once (asse_bytes.h).
+// special case.
 #pragma once
 
 #include <cstdint>

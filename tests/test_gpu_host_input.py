@@ -22,9 +22,11 @@ def mods():
 
 
 @pytest.mark.parametrize("max_batch,pinned,sizes", [
-    (0, True, (2 * MI - 1, 2 * MI, 2 * MI + 1, 1)),         # unsplit, split even and odd, a lone pair
+    (0, True, (2 * MI - 1, 2 * MI, 2 * MI + 1, 1)),         # two parts of one chunk, even and odd, a lone pair
+    (0, True, (5 * MI // 4, 5 * MI // 4 + 1, MI + 1)),      # one part, two parts, one part
     (0, True, (4 * MI, 4 * MI + 1, 6 * MI + 3, 9 * MI + 5)),  # one, two and three chunks, the last one short, split or not
-    (3 * MI - 1, True, (3 * MI, 6 * MI + 1, 5 * MI + 7)),   # a buffer of an odd size
+    (3 * MI - 1, True, (3 * MI, 6 * MI + 1, 5 * MI + 7)),   # a buffer of an odd size; halves, whole buffers
+    (65_001, True, (5 * MI // 4 + 3, 131_072, 65_003)),     # a buffer smaller than the parts and their alignment
     (0, False, (2 * MI + 1, 5 * MI + 3)),                    # pageable memory
     (1, True, (1, 2, 7))])
 def test_host_chunks_equal_device_input(mods, max_batch, pinned, sizes):
