@@ -40,11 +40,12 @@ MLP_FLOP_PER_ROW = 2 * (68 * 256 + 256 * 256 + 256)
 # A figure whose source id no longer matches the current sources is reported
 # as null (the kernel has changed since the capture).
 TRAFFIC = {
-    ("long", "hist", "ingest"): (1295601920, "d0191276ba84"),
-    ("long", "hist", "hist_scan"): (147243248, "bd35d6abdfed"),
-    ("link", "at", "ingest"): (201379072, "d0191276ba84"),
-    ("link", "at", "scan"): (96883456, "7fe98d3eebca"),
-    ("long", "at", "scan"): (1081540752, "7fe98d3eebca"),
+    ("long", "hist", "ingest"): (1295525368, "84ac5f23dccf"),
+    ("long", "hist", "hist_scan"): (146776672, "b1ab32627ee9"),
+    ("link", "at", "ingest"): (204297216, "84ac5f23dccf"),
+    ("link", "at", "scan"): (95505920, "0c3116953443"),
+    ("long", "at", "ingest"): (747020944, "84ac5f23dccf"),
+    ("long", "at", "scan"): (1079074784, "0c3116953443"),
 }
 KERNEL_SOURCES = {
     "ingest": ["asse_ingest.cu", "asse_device.cuh", "asse_internal.h"],
@@ -945,7 +946,7 @@ def main():
     ap.add_argument("--cycled", type=int, default=0,
                     help="distinct input slices cycled through (0: 8, or 4 for slices over 8 Mi pairs)")
     ap.add_argument("--key-table", default="auto", choices=["auto", "on", "off"],
-                    help="the ingest's slice-wide key table (auto: for pools larger than L2)")
+                    help="the ingest's slice-wide key table (auto: for every pool but those with slice counts that fit in L2)")
     ap.add_argument("--clocks-dir", default="", help="where the nvidia-smi clock samples of the timed region go "
                                                       "(default: the temporary directory)")
     ap.add_argument("--counter", default="auto", choices=["auto", "at", "ace", "aligned", "hist"],

@@ -44,6 +44,10 @@ ASSE_API uint64_t asse_server_bytes_in_use(const asse_server *srv);
  * (synchronises).  Returns ASSE_ENOMEM, without side effects, if the stream
  * does not fit the budget next to the open streams: the caller retries after
  * asse_server_close frees memory.  *id receives the stream id.
+ * With key_table ASSE_KEYS_AUTO the pool keeps a key table only where it is
+ * larger than the device's L2 cache; ASSE_KEYS_ON gives a smaller one a table
+ * too, charged to the budget, which makes its ingest faster unless its slices
+ * have many more distinct pairs than the pool has ATs (asse.h).
  * Errors: EINVAL, ENOMEM, ECUDA. */
 ASSE_API int asse_server_open(asse_server *srv, const asse_config *cfg, uint32_t kp, uint64_t max_batch,
                               uint32_t *id);

@@ -13,15 +13,17 @@
 // keys new to the slice go on, through a second per-warp queue, to Algorithm 3:
 // each lane takes one, computes f(aip), the frame, the r column indices and the
 // ACT of the AT in registers, then sets the r fields without reading them.
-// Without a key table the r words are read together first, and a field that
+// Without a key table, and in dense slices (claim_pairs, blind_pairs in
+// asse_api.cu), the r words are read together first, and a field that
 // already holds the slice's value costs one load and no atomic.  Across the
 // 152 blocks a hot key reaches the pool once instead of once per block.  What
-// bounds the launch is the number of requests the L2 serves (the link pool,
-// 92 MB: 12 M of them in 89 us, against 22 M in 103 us without a table; loads
-// mixed with atomics go at about 135 G a second there) and, for a pool in HBM,
-// DRAM's random accesses.  The seen table is 64 KB: with 128 KB the launch also
-// empties a larger table (6.2 -> 7.2 us for 65,536 pairs) and, where pool words
-// are read, leaves less L1 for them.
+// bounds the launch is the number of requests the L2 serves (the link workload's
+// slice, 8 Mi pairs on a 92 MB pool: 12.7 M requests in 84 us, 104 us without a
+// table) and, for a pool in HBM, DRAM's random accesses.  The seen table is
+// 64 KB: with 128 KB, 65,536 pairs on a 0.5 MB pool take 15.4 us instead of 14.2
+// (from event to event), as the launch empties a larger table, and the long
+// workload's slices with slice counts 414 instead of 386, as the pool words that
+// are read have less L1 (timestamps alone: 312 / 318).
 #include <cooperative_groups.h>
 #include <cuda_runtime.h>
 
@@ -80,9 +82,9 @@ constexpr uint32_t NO_AIP = 0;      // marks an empty way; a pair of this addres
 // exactly and a way holds the 32 bits of aip alone: twice the keys of 64-bit
 // entries.  Two ways, the newer first, the older pushed out.  By a model of the
 // tables, of the 33.5 M pairs of a slice of the long workload 10.1 M miss it
-// (11.5 M missed a direct-mapped table of 64-bit entries of the same 64 KB, and
-// 9.5 M would miss 128 KB); measured, the long ingest runs in 247 us (315 us
-// direct-mapped, 251 us with 128 KB), with slice counts in 374 us (382, 406).
+// (11.5 M missed a direct-mapped table of 64-bit entries of the same 64 KB);
+// measured, medians over five such inputs, its ingest takes 318 us (316
+// direct-mapped), with slice counts 386 (390).
 // Without CLUSTER: the block's own table.
 // With it: the 2^cl_log2 CTAs of a thread-block cluster share one table, each
 // CTA holding the sets whose top bits pick it, reached by the others through
@@ -221,8 +223,8 @@ enum SetKind {
 // 92 MB buffer.  A byte field is stored; narrower fields take one atomicAnd
 // that clears the bits outside the value and one atomicOr that sets those
 // inside.  All writers of a field within a slice write the same value, so
-// every interleaving ends at it.  Measured (33.5 M pairs, 1.07 GB pool): 349 ->
-// 314 us; 8.4 M pairs on a 92 MB pool with a key table: 114 -> 93 us.  The
+// every interleaving ends at it.  Measured (33.5 M pairs, 1.07 GB pool): 362 ->
+// 317 us; 8.4 M pairs on a 92 MB pool with a key table: 118 -> 86 us.  The
 // slice counts need the old value and keep reading: taking it from an atomicOr
 // that also sets the byte's guard bit as a marker of a change in progress ran
 // 431 against 382 us.
