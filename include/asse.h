@@ -307,8 +307,9 @@ ASSE_API int asse_estimate(asse_pool *pool, const uint32_t *aips, uint64_t n, as
  * 4,096 entries waits only for that close or restore (work queued on the stream
  * after it, such as asse_advance or the next batch's ingest, keeps running);
  * otherwise the call synchronises the stream after its copy, so that out may be
- * read on any stream.  After a restore or close that the caller captured into a
- * graph, it synchronises the stream first, which the graph is launched on.
+ * read on any stream.  Once a restore or close of the pool has been captured into
+ * a graph of the caller's, every read synchronises the pool's stream, on which the
+ * graph is to be launched.
  * Returns ECAPACITY if cap < count, or
  * if the restore overflowed restore_cap (then *n_out is the number of
  * column tuples the overflowing join level needed, a lower bound on the

@@ -809,7 +809,8 @@ int asse_ingest(asse_pool *p, const uint32_t *pairs, uint64_t n, int where)
         return fail(p, ASSE_EINVAL, "where must be ASSE_HOST or ASSE_DEVICE");
     if (where == ASSE_DEVICE && ((uintptr_t)pairs & 15) != 0)
         return fail(p, ASSE_EINVAL, "device pairs must be 16-byte aligned");
-    p->slice_pairs += n;
+    // (a captured close opens slices that the host does not see)
+    p->slice_pairs = p->captured ? n : p->slice_pairs + n;
     Params P = p->P;
     if (p->slice_pairs > p->claim_pairs)
         P.keys = nullptr;
